@@ -87,18 +87,22 @@ inline PointwiseArgsT<T> cast_args(const PointwiseArgs& a) {
 // A row-major M x K (lda), B row-major K x N (ldb), C/base/base2 row-major
 // M x N (ldc).  *_bs are batch strides in elements.
 struct GemmArgs {
-  const void* A[2];
-  const void* B[2];
-  void* C[2];
-  const void* base[2];
-  const void* base2[2];
+  const void* A[4];
+  const void* B[4];
+  void* C[4];
+  const void* base[4];
+  const void* base2[4];
   int64_t lda, ldb, ldc;
   int64_t a_bs, b_bs, c_bs;
   int M, N, K;
   int batch;   // p range
-  int ncomp;   // 1 or 2
+  int ncomp;   // 1 to 4
   double alpha, beta, beta2;
 };
+
+// Programmatic dependent launch for the kernels of a step (ADR_PDL=0 turns
+// it off: every kernel then waits for the previous one to finish).
+bool pdl_enabled();
 
 // Kernel launchers (simt.cu).
 template <typename T>

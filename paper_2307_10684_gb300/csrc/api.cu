@@ -103,6 +103,16 @@ static bool same_operator(const Tridiag& a, const Tridiag& b) {
   return a.lo == b.lo && a.di == b.di && a.up == b.up && a.b0 == b.b0 && a.bn == b.bn;
 }
 
+namespace adr {
+bool pdl_enabled() {
+  static const int on = [] {
+    const char* e = getenv("ADR_PDL");
+    return e ? atoi(e) : 1;
+  }();
+  return on != 0;
+}
+}  // namespace adr
+
 // ---------------------------------------------------------------- step (SIMT)
 template <typename T>
 static cudaError_t mode_product_simt(adr_plan P, int mu, int ell, void* const in[2], void* const out[2],
@@ -118,7 +128,6 @@ static cudaError_t mode_product_simt(adr_plan P, int mu, int ell, void* const in
   for (int c = 0; c < 2; ++c) {
     g.C[c] = out[c];
     g.base[c] = base ? base[c] : nullptr;
-    g.base2[c] = nullptr;
   }
   if (mu == 0) {  // Y[p][i] = sum_j X[p][j] Phi[i][j]  ->  Y = X Phi^T
     for (int c = 0; c < 2; ++c) {

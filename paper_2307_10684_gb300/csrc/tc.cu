@@ -431,14 +431,49 @@ __device__ __forceinline__ void comp_update(float b, float lo_in, float inc, flo
 
 __device__ __forceinline__ double trap_w(int i, int n) { return (i == 0 || i == n - 1) ? 0.5 : 1.0; }
 
+// Indicator sums (Sec. 4) of one lane's values: sum of w x and of (x - x_prev)^2,
+// kept as FP32 pairs by TwoSum (about 48 bits) and not in FP64: the FP64 pipe
+// retires two operations a clock and SM, and five per value took 40 us of the
+// last product of a 200^2 grid (58 of 118 us a step; 46 with the pairs).
+struct IndSums {
+  float sh = 0.f, sl = 0.f, dh = 0.f, dl = 0.f;
+  static __device__ __forceinline__ void acc(float& h, float& l, float x) {
+    float s, e;
+    two_sum(h, x, s, e);
+    h = s;
+    l = __fadd_rn(l, e);
+  }
+  __device__ __forceinline__ void add(float x, float prev, bool edge) {
+    acc(sh, sl, edge ? 0.5f * x : x);
+    float d, de;  // x - prev, exactly d + de
+    two_sum(x, -prev, d, de);
+    const float p = __fmul_rn(d, d);
+    acc(dh, dl, p);
+    dl = __fadd_rn(dl, __fmaf_rn(__fmul_rn(2.f, d), de, __fmaf_rn(d, d, -p)));
+  }
+  // adds the warp's sums (lane weight wm) to the step's slot
+  __device__ __forceinline__ void flush(double wm, double* ind) const {
+    double sw = wm * ((double)sh + (double)sl), sd = (double)dh + (double)dl;
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      sw += __shfl_xor_sync(0xffffffffu, sw, off);
+      sd += __shfl_xor_sync(0xffffffffu, sd, off);
+    }
+    if ((threadIdx.x & 31) == 0) {
+      atomicAdd(ind, sw);
+      atomicAdd(ind + 2, sd);
+    }
+  }
+};
+
 // Epilogue of a kAxpy pass with its options, for one epilogue warp: lane =
 // output row m, NCH chunks of 16 columns from n0; out = base + alpha acc.
 //  lp  : compensated state; the low-order words are read and rewritten in
 //        place and hi + lo takes the exact sum (comp_update).
 //  ind : the step's indicator slot of this component: adds the
 //        trapezoid-weighted sum of the new state and the squared increment
-//        against the value the output buffer held (the previous state), in
-//        FP64, one atomic per warp and sum.
+//        against the value the output buffer held (the previous state), one
+//        FP64 atomic per warp and sum.
 // Per chunk the base, low-order and previous values are loaded before the
 // TMEM read, so their latency overlaps it.
 template <int NCH>
@@ -448,7 +483,7 @@ __device__ __forceinline__ void axpy_epilogue(uint32_t ta, float* __restrict__ o
                                               double* ind, int n1, int n2) {
   double wm = 0.0;  // trapezoid weight of row m (the directions before the last)
   if (ind && mrow) wm = n2 > 0 ? trap_w(m % n1, n1) * trap_w(m / n1, n2) : trap_w(m, n1);
-  double sw = 0.0, sd = 0.0;
+  IndSums sums;
 #pragma unroll 1
   for (int bt = 0; bt < NCH; ++bt) {
     float bb[16], lv[16], pv[16];
@@ -480,25 +515,11 @@ __device__ __forceinline__ void axpy_epilogue(uint32_t ta, float* __restrict__ o
           hi = __fmaf_rn(alpha, a, bb[jj]);
         }
         of[o] = hi;
-        if (ind) {
-          sw += wm * trap_w(col, N) * (double)hi;
-          const double dd = (double)hi - (double)pv[jj];
-          sd += dd * dd;
-        }
+        if (ind) sums.add(hi, pv[jj], col == 0 || col == N - 1);
       }
     }
   }
-  if (ind) {
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-      sw += __shfl_xor_sync(0xffffffffu, sw, off);
-      sd += __shfl_xor_sync(0xffffffffu, sd, off);
-    }
-    if ((threadIdx.x & 31) == 0) {
-      atomicAdd(ind, sw);
-      atomicAdd(ind + 2, sd);
-    }
-  }
+  if (ind) sums.flush(wm, ind);
 }
 
 // The indicator slot of component c for the unit's step (null when off).
@@ -1530,10 +1551,10 @@ __device__ __forceinline__ void split3_pair(float x0, float x1, uint32_t& w0, ui
   const float r0 = x0 - f0.x, r1 = x1 - f0.y;
   const __nv_bfloat162 h1 = __floats2bfloat162_rn(r0, r1);
   const float2 f1 = __bfloat1622float2(h1);
-  const __nv_bfloat162 h2 = __floats2bfloat162_rn(r0 - f1.x, r1 - f1.y);
+  const __nv_bfloat162 tp = __floats2bfloat162_rn(r0 - f1.x, r1 - f1.y);
   w0 = *reinterpret_cast<const uint32_t*>(&h0);
   w1 = *reinterpret_cast<const uint32_t*>(&h1);
-  w2 = *reinterpret_cast<const uint32_t*>(&h2);
+  w2 = *reinterpret_cast<const uint32_t*>(&tp);
 }
 static_assert(2 * kPieces * kFTileC <= kFStage, "an MMA2 stage fits in a ring slot");
 static_assert(kFSmem <= 227 * 1024, "shared memory per CTA");
@@ -2003,6 +2024,8 @@ struct PwLaunch {
   const int* bstart;   // [nsolves + 1] prefix sums of this kernel's blocks (desc non-null)
   int nsolves;
   int* err;            // device error word (bounded waits)
+  uint32_t* ctl;       // claims and counters of the two-pass launch that follows (or null),
+  int nctl;            // cleared here
 };
 
 constexpr int kPwThreads = 256;
@@ -2017,13 +2040,26 @@ constexpr int kFlatPerBlock = kPwThreads * 4 * kFlatVec;
 // static; the data it points to is not).
 // home = the descriptor where it lives (launch parameter or device memory),
 // from where tensor maps must be read.
+// The next kernel is let in at once; if it is a two-pass launch, only when
+// the previous operator is complete and its claims and counters are cleared,
+// because it claims units before this kernel has finished.
+__device__ __forceinline__ void pw_open(const PwLaunch& L) {
+  pdl_wait();
+  if (L.ctl == nullptr) return;
+  if (blockIdx.x == 0) {
+    for (int i = threadIdx.x; i < L.nctl; i += blockDim.x) L.ctl[i] = 0u;
+    __threadfence();
+    __syncthreads();
+  }
+  pdl_trigger();
+}
 __device__ __forceinline__ const PwDesc* block_desc(const PwLaunch& L, PwDesc* sd, int& lb,
                                                     const PwDesc** home = nullptr) {
-  pdl_trigger();
+  if (L.ctl == nullptr) pdl_trigger();
   if (L.desc == nullptr) {
     lb = blockIdx.x;
     if (home) *home = &L.one;
-    pdl_wait();
+    pw_open(L);
     return &L.one;
   }
   const int s = find_segment(L.bstart, L.nsolves, blockIdx.x);
@@ -2034,7 +2070,7 @@ __device__ __forceinline__ const PwDesc* block_desc(const PwLaunch& L, PwDesc* s
   for (int w = threadIdx.x; w < (int)(sizeof(PwDesc) / 4); w += blockDim.x) dst[w] = __ldg(src + w);
   lb = blockIdx.x - __ldg(L.bstart + s);
   __syncthreads();
-  pdl_wait();
+  pw_open(L);
   return sd;
 }
 
@@ -2153,7 +2189,7 @@ __global__ void __launch_bounds__(kPwThreads, 2) rhs_pieces_kernel(const __grid_
   // axis coefficients: x = mu 1, z = mu 2
   const Coef cxu = coef(dp->a.A[0][0]), cxv = coef(dp->a.A[1][0]);
   const Coef czu = coef(dp->a.A[0][1]), czv = coef(dp->a.A[1][1]);
-  const ReactionT<float> rx = dp->a.rx;
+  const ReactionT<float>& rx = dp->a.rx;
   const int64_t col = x0;
   const float4 zero4 = make_float4(0.f, 0.f, 0.f, 0.f);
   // run ends: lane 0 needs x0 - 1, lane 31 needs x0 + 4 (others come by shuffle)
@@ -2195,11 +2231,15 @@ __global__ void __launch_bounds__(kPwThreads, 2) rhs_pieces_kernel(const __grid_
         ur = eu[q];
         vr = ev[q];
       }
-      float ou[4], ov[4];
+      // the stencil of four points, then their reactions with the model's
+      // switch outside the points (for_model)
+      float cu[4], cv[4], ou[4], ov[4];
+      dfloat du[DF ? 4 : 1], dv[DF ? 4 : 1];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
         const int xi = x0 + j;
-        const float cu = el(uc, j), cv = el(vc, j);
+        cu[j] = el(uc, j);
+        cv[j] = el(vc, j);
         const float lu = j == 0 ? ul : el(uc, j - 1), lv = j == 0 ? vl : el(vc, j - 1);
         const float ru = j == 3 ? ur : el(uc, j + 1), rv = j == 3 ? vr : el(vc, j + 1);
         if constexpr (DF) {  // accurate mode: stencil and reaction in double-float, one rounding
@@ -2207,25 +2247,30 @@ __global__ void __launch_bounds__(kPwThreads, 2) rhs_pieces_kernel(const __grid_
           const CoefDF dxv = coef_df(dp->a.A[1][0], dp->a.Alo[1][0]);
           const CoefDF dzu = coef_df(dp->a.A[0][1], dp->a.Alo[0][1]);
           const CoefDF dzv = coef_df(dp->a.A[1][1], dp->a.Alo[1][1]);
-          dfloat gu, gv;
-          react_dfd(rx, cu, cv, gu, gv);
-          ou[j] = df_round(dtri_x4(j, lu, cu, ru, xi, nx, dxu.lo, dxu.up, dxu.b0, dxu.bn) +
-                           dtri_dir(el(pu[q], j), cu, el(pu[q + 2], j), zq, nz, dzu.lo, dzu.up,
-                                    dzu.b0, dzu.bn) + gu);
-          ov[j] = df_round(dtri_x4(j, lv, cv, rv, xi, nx, dxv.lo, dxv.up, dxv.b0, dxv.bn) +
-                           dtri_dir(el(pv[q], j), cv, el(pv[q + 2], j), zq, nz, dzv.lo, dzv.up,
-                                    dzv.b0, dzv.bn) + gv);
+          du[j] = dtri_x4(j, lu, cu[j], ru, xi, nx, dxu.lo, dxu.up, dxu.b0, dxu.bn) +
+                  dtri_dir(el(pu[q], j), cu[j], el(pu[q + 2], j), zq, nz, dzu.lo, dzu.up, dzu.b0, dzu.bn);
+          dv[j] = dtri_x4(j, lv, cv[j], rv, xi, nx, dxv.lo, dxv.up, dxv.b0, dxv.bn) +
+                  dtri_dir(el(pv[q], j), cv[j], el(pv[q + 2], j), zq, nz, dzv.lo, dzv.up, dzv.b0, dzv.bn);
         } else {
-          float ku = tri_x4(j, lu, cu, ru, xi, nx, cxu.lo, cxu.up, cxu.b0, cxu.bn);
-          float kv = tri_x4(j, lv, cv, rv, xi, nx, cxv.lo, cxv.up, cxv.b0, cxv.bn);
-          ku += tri_dir(el(pu[q], j), cu, el(pu[q + 2], j), zq, nz, czu.lo, czu.up, czu.b0, czu.bn);
-          kv += tri_dir(el(pv[q], j), cv, el(pv[q + 2], j), zq, nz, czv.lo, czv.up, czv.b0, czv.bn);
-          float gu, gv;
-          react<float>(rx, cu, cv, gu, gv);
-          ou[j] = ku + gu;
-          ov[j] = kv + gv;
+          ou[j] = tri_x4(j, lu, cu[j], ru, xi, nx, cxu.lo, cxu.up, cxu.b0, cxu.bn) +
+                  tri_dir(el(pu[q], j), cu[j], el(pu[q + 2], j), zq, nz, czu.lo, czu.up, czu.b0, czu.bn);
+          ov[j] = tri_x4(j, lv, cv[j], rv, xi, nx, cxv.lo, cxv.up, cxv.b0, cxv.bn) +
+                  tri_dir(el(pv[q], j), cv[j], el(pv[q + 2], j), zq, nz, czv.lo, czv.up, czv.b0, czv.bn);
         }
       }
+      for_model<4>(rx, [&](const ReactionT<float>& r, int j) {
+        if constexpr (DF) {
+          dfloat gu, gv;
+          react_dfd(r, cu[j], cv[j], gu, gv);
+          ou[j] = df_round(du[j] + gu);
+          ov[j] = df_round(dv[j] + gv);
+        } else {
+          float gu, gv;
+          react<float>(r, cu[j], cv[j], gu, gv);
+          ou[j] += gu;
+          ov[j] += gv;
+        }
+      });
       if (act) {
         const int64_t idx = (int64_t)zq * sz + col;
         store_pieces_fmt<F>(wu, N, idx, ou);
@@ -2428,7 +2473,7 @@ constexpr int kZB2 = 4;  // planes per iteration of the 2D stencil kernel
 template <int F = kFmtBF16>
 __global__ void __launch_bounds__(kPwThreads) rdiff_pieces_kernel(const __grid_constant__ PwLaunch L) {
   FLAT_PROLOGUE
-  const ReactionT<float> rx = sd.a.rx;
+  const ReactionT<float>& rx = sd.a.rx;
   float4 a0[kFlatVec], a1[kFlatVec], a2[kFlatVec], a3[kFlatVec];
 #pragma unroll
   for (int k = 0; k < kFlatVec; ++k) {
@@ -2444,13 +2489,12 @@ __global__ void __launch_bounds__(kPwThreads) rdiff_pieces_kernel(const __grid_c
   for (int k = 0; k < kFlatVec; ++k) {
     const int64_t g = g0 + k * kPwThreads;
     if (g >= N4) break;
+    // the increment form (react_diff) in both modes: its rounding is
+    // relative to the difference itself
     float du[4], dv[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-      // the increment form (react_diff) in both modes: its rounding is
-      // relative to the difference itself
-      react_diff<float>(rx, el(a0[k], j), el(a1[k], j), el(a2[k], j), el(a3[k], j), du[j], dv[j]);
-    }
+    for_model<4>(rx, [&](const ReactionT<float>& r, int j) {
+      react_diff<float>(r, el(a0[k], j), el(a1[k], j), el(a2[k], j), el(a3[k], j), du[j], dv[j]);
+    });
     store_pieces_fmt<F>(sd.wu, N, 4 * g, du);
     store_pieces_fmt<F>(sd.wv, N, 4 * g, dv);
   }
@@ -2462,7 +2506,7 @@ template <int F = kFmtBF16>
 __global__ void __launch_bounds__(kPwThreads) lawson_pre_pieces_kernel(const __grid_constant__ PwLaunch L,
                                                                        float factor) {
   FLAT_PROLOGUE
-  const ReactionT<float> rx = sd.a.rx;
+  const ReactionT<float>& rx = sd.a.rx;
   const float sc = factor * sd.tau;
   float4 a0[kFlatVec], a1[kFlatVec];
 #pragma unroll
@@ -2478,14 +2522,13 @@ __global__ void __launch_bounds__(kPwThreads) lawson_pre_pieces_kernel(const __g
     const int64_t g = g0 + k * kPwThreads;
     if (g >= N4) break;
     float wu[4], wv[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for_model<4>(rx, [&](const ReactionT<float>& r, int j) {
       const float uu = el(a0[k], j), vv = el(a1[k], j);
       float gu, gv;
-      react<float>(rx, uu, vv, gu, gv);
+      react<float>(r, uu, vv, gu, gv);
       wu[j] = uu + sc * gu;
       wv[j] = vv + sc * gv;
-    }
+    });
     store_pieces_fmt<F>(sd.wu, N, 4 * g, wu);
     store_pieces_fmt<F>(sd.wv, N, 4 * g, wv);
   }
@@ -2494,7 +2537,7 @@ __global__ void __launch_bounds__(kPwThreads) lawson_pre_pieces_kernel(const __g
 // Lawson2b last stage: u += factor tau G(u2, v2) in FP32, in place.
 __global__ void __launch_bounds__(kPwThreads) lawson_post_kernel(const __grid_constant__ PwLaunch L, float factor) {
   FLAT_PROLOGUE
-  const ReactionT<float> rx = sd.a.rx;
+  const ReactionT<float>& rx = sd.a.rx;
   const float sc = factor * sd.tau;
   float* u = const_cast<float*>(sd.u);
   float* v = const_cast<float*>(sd.v);
@@ -2514,13 +2557,12 @@ __global__ void __launch_bounds__(kPwThreads) lawson_post_kernel(const __grid_co
     const int64_t g = g0 + k * kPwThreads;
     if (g >= N4) break;
     float ou[4], ov[4];
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
+    for_model<4>(rx, [&](const ReactionT<float>& r, int j) {
       float gu, gv;
-      react<float>(rx, el(a0[k], j), el(a1[k], j), gu, gv);
+      react<float>(r, el(a0[k], j), el(a1[k], j), gu, gv);
       ou[j] = el(a2[k], j) + sc * gu;
       ov[j] = el(a3[k], j) + sc * gv;
-    }
+    });
     *reinterpret_cast<float4*>(u + 4 * g) = make_float4(ou[0], ou[1], ou[2], ou[3]);
     *reinterpret_cast<float4*>(v + 4 * g) = make_float4(ov[0], ov[1], ov[2], ov[3]);
   }
@@ -2634,6 +2676,8 @@ __global__ void __launch_bounds__(32 * kBandWarps) band_support_kernel(
   if (threadIdx.x == 0) band[blockIdx.x] = make_int2(s_lo & ~63, min(n, (s_hi + 63) & ~63));
 }
 
+#include "twopass.cuh"
+
 // ---------------------------------------------------------------- host side
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
 
@@ -2681,6 +2725,19 @@ cudaError_t encode_pieces_mn(CUtensorMap* map, const void* base, int64_t M, int6
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// [3][rows][K] BF16 pieces, box {32, box_rows, pieces}, 64-byte swizzle (the
+// two-pass launch loads Phi one piece at a time on tiles below 128 rows).
+cudaError_t encode_tp(CUtensorMap* map, const void* base, int64_t K, int64_t rows, int box_rows, int pieces) {
+  cuuint64_t dims[3] = {(cuuint64_t)K, (cuuint64_t)rows, (cuuint64_t)kPieces};
+  cuuint64_t strides[2] = {(cuuint64_t)K * 2, (cuuint64_t)(K * rows) * 2};
+  cuuint32_t box[3] = {(cuuint32_t)kTpBK, (cuuint32_t)box_rows, (cuuint32_t)pieces};
+  cuuint32_t estr[3] = {1, 1, 1};
+  CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims,
+                        strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
+                        CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
 // Kernel variants (swizzle width, tile width, CTA pair).  Pair variants run
 // tc_pair_kernel: 256-row tiles over two SMs.
 struct Variant {
@@ -2714,16 +2771,6 @@ cudaError_t set_smem_attr_pair() {
     e = cudaFuncSetAttribute(tc_pair_kernel<SW, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              Tc2Cfg<SW>::SMEM);
   return e;
-}
-
-// Programmatic dependent launch for the kernels of a step (ADR_PDL=0 turns
-// it off: every kernel then waits for the previous one to finish).
-static bool pdl_enabled() {
-  static const int on = [] {
-    const char* e = getenv("ADR_PDL");
-    return e ? atoi(e) : 1;
-  }();
-  return on != 0;
 }
 
 template <typename... KArgs, typename... Args>
@@ -2899,6 +2946,59 @@ cudaError_t launch_fused(int slots, cudaStream_t s, const TcLaunch& L, bool ind)
   return launch_k(tc_fused_kernel<false>, grid, dim3(kThreads), kFSmem, s, L);
 }
 
+// The two-pass launch, and (amn) the x3 product after it; bn: its widest tile.
+template <bool AMN, bool WIDE>
+cudaError_t launch_tp_t(int sms, cudaStream_t s, const TpLaunch& L, int epi) {
+  const dim3 grid((unsigned)std::min(L.nunits, sms)), block(kTpThreads);
+  constexpr int smem = TpCfg<WIDE>::SMEM;
+  if (epi == 2) return launch_k(tp_kernel<2, AMN, WIDE>, grid, block, smem, s, L);
+  if (epi == 1) return launch_k(tp_kernel<1, AMN, WIDE>, grid, block, smem, s, L);
+  return launch_k(tp_kernel<0, AMN, WIDE>, grid, block, smem, s, L);
+}
+cudaError_t launch_tp(int sms, cudaStream_t s, TpLaunch& L, bool amn, int bn, int epi) {
+  if (L.nunits <= 0) return cudaSuccess;
+  L.ahead = L.nunits >= 16 * sms ? 3 : (L.nunits >= 6 * sms ? 1 : 0);
+  if (bn > 128) return amn ? launch_tp_t<true, true>(sms, s, L, epi) : launch_tp_t<false, true>(sms, s, L, epi);
+  return amn ? launch_tp_t<true, false>(sms, s, L, epi) : launch_tp_t<false, false>(sms, s, L, epi);
+}
+// 3D stencil on whole rows (nseg: 64-point segments of the widest row).
+template <bool DF>
+cudaError_t launch_rhs3_rows(int nseg, int blocks, cudaStream_t s, const PwLaunch& L) {
+  const dim3 g(blocks), b(kPwThreads);
+  if (nseg == 1) return launch_k(rhs3_row_kernel<1, DF>, g, b, kRowRingSmem, s, L);
+  if (nseg == 2) return launch_k(rhs3_row_kernel<2, DF>, g, b, kRowRingSmem, s, L);
+  if (nseg == 3) return launch_k(rhs3_row_kernel<3, DF>, g, b, kRowRingSmem, s, L);
+  return launch_k(rhs3_row_kernel<4, DF>, g, b, kRowRingSmem, s, L);
+}
+cudaError_t set_tp_attr() {
+  const auto at = cudaFuncAttributeMaxDynamicSharedMemorySize;
+  cudaError_t e = cudaSuccess;
+  auto set = [&](auto* f, int sm) {
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(f, at, sm);
+  };
+  set(tp_kernel<0, false, false>, TpCfg<false>::SMEM);
+  set(tp_kernel<0, false, true>, TpCfg<true>::SMEM);
+  set(tp_kernel<0, true, false>, TpCfg<false>::SMEM);
+  set(tp_kernel<0, true, true>, TpCfg<true>::SMEM);
+  set(tp_kernel<1, false, false>, TpCfg<false>::SMEM);
+  set(tp_kernel<1, false, true>, TpCfg<true>::SMEM);
+  set(tp_kernel<1, true, false>, TpCfg<false>::SMEM);
+  set(tp_kernel<1, true, true>, TpCfg<true>::SMEM);
+  set(tp_kernel<2, false, false>, TpCfg<false>::SMEM);
+  set(tp_kernel<2, false, true>, TpCfg<true>::SMEM);
+  set(tp_kernel<2, true, false>, TpCfg<false>::SMEM);
+  set(tp_kernel<2, true, true>, TpCfg<true>::SMEM);
+  set(rhs3_row_kernel<1, false>, kRowRingSmem);
+  set(rhs3_row_kernel<2, false>, kRowRingSmem);
+  set(rhs3_row_kernel<3, false>, kRowRingSmem);
+  set(rhs3_row_kernel<4, false>, kRowRingSmem);
+  set(rhs3_row_kernel<1, true>, kRowRingSmem);
+  set(rhs3_row_kernel<2, true>, kRowRingSmem);
+  set(rhs3_row_kernel<3, true>, kRowRingSmem);
+  set(rhs3_row_kernel<4, true>, kRowRingSmem);
+  return e;
+}
+
 int grid_for(int64_t total) {
   int64_t b = (total + 255) / 256;
   if (b < 1) b = 1;
@@ -2919,6 +3019,7 @@ struct TcPass {
   int out, base, alpha;
   int fused;  // 1: modes 1 and 2 in one launch (tc_fused_kernel); mu = 0
   int amn;    // 1: reads the fused pass's natural-layout pieces as an MN-major A (mu = 2)
+  int tp;     // tp_kernel: the x1 and x2 products as dependent passes (fused), or the x3 product after them
 };
 
 // One launch of the step sequence.
@@ -2986,6 +3087,11 @@ struct TcState {
   // sums (w u, w v, |dU|^2, |dV|^2) and the step counter
   double* ind;
   int64_t* ind_ctr;
+  // two-pass launches (twopass.cuh)
+  int tp;
+  __nv_bfloat16* mid[2];                  // 3D: output pieces of the two-pass launch
+  uint32_t* tpctl;                        // its claims and dependency counters
+  std::vector<TpOp> h_op;                 // [passes]
 };
 
 static int units_of(const TcState* S, const TcPass& ps, int bn) {
@@ -3074,7 +3180,11 @@ struct PwGeom {
   int nx, ny, nz, xsegs, ytiles, zlen, zsegs;
   int64_t sy, sz;
 };
-static PwGeom pw_geom(const TcState* S, int num_sms, double share) {
+// The 3D stencil on whole rows (rhs3_row_kernel; in a batch, if every solve's
+// rows are short enough).  us a launch, rhs3_ring_kernel / this one: 160^3
+// accurate mode 132 / 94, plain 45 / 40; 256^3 plain 99 / 101.
+static bool row_ring(const TcState* S) { return S->d == 3 && S->fmt == kFmtBF16 && S->n[0] <= 192; }
+static PwGeom pw_geom(const TcState* S, int num_sms, double share, bool ring) {
   PwGeom g;
   const bool d3 = S->d == 3;
   g.nx = (int)S->n[0];
@@ -3083,8 +3193,8 @@ static PwGeom pw_geom(const TcState* S, int num_sms, double share) {
     g.ny = (int)S->n[1];
     g.nz = (int)S->n[2];
     g.sz = S->n[0] * S->n[1];
-    g.xsegs = (g.nx + kRingX - 1) / kRingX;
-    g.ytiles = (g.ny + kRingY - 1) / kRingY;
+    g.xsegs = ring ? 1 : (g.nx + kRingX - 1) / kRingX;
+    g.ytiles = ring ? (g.ny + kRowRingY - 1) / kRowRingY : (g.ny + kRingY - 1) / kRingY;
     const int64_t cols = (int64_t)g.xsegs * g.ytiles;
     const int64_t want = std::max<int64_t>(1, (int64_t)(num_sms * 2 * 2 * share + 0.5));
     int64_t segs = (want + cols - 1) / cols;
@@ -3116,11 +3226,12 @@ static PwGeom pw_geom(const TcState* S, int num_sms, double share) {
 }
 
 // 3D state field [nz][ny][nx] FP32 for the stencil's plane copies: box
-// {kRingBoxX, kRingBoxY, 1}, zero fill outside the grid.
-static cudaError_t encode_field(CUtensorMap* map, const float* base, const PwGeom& g) {
+// {kRingBoxX, kRingBoxY, 1} (ring: whole rows, kRowRingY + 2 of them), zero
+// fill outside the grid.
+static cudaError_t encode_field(CUtensorMap* map, const float* base, const PwGeom& g, bool ring) {
   cuuint64_t dims[3] = {(cuuint64_t)g.nx, (cuuint64_t)g.ny, (cuuint64_t)g.nz};
   cuuint64_t strides[2] = {(cuuint64_t)g.sy * 4, (cuuint64_t)g.sz * 4};
-  cuuint32_t box[3] = {(cuuint32_t)kRingBoxX, (cuuint32_t)kRingBoxY, 1};
+  cuuint32_t box[3] = {(cuuint32_t)(ring ? g.nx : kRingBoxX), (cuuint32_t)(ring ? kRowRingY + 2 : kRingBoxY), 1};
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = g_encode(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 3, const_cast<float*>(base), dims,
                         strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE,
@@ -3128,7 +3239,7 @@ static cudaError_t encode_field(CUtensorMap* map, const float* base, const PwGeo
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-static cudaError_t make_pw(const TcState* S, const adr_plan_s* P, float* u, float* v, PwDesc* out,
+static cudaError_t make_pw(const TcState* S, const adr_plan_s* P, float* u, float* v, PwDesc* out, bool ring,
                            double share = 1.0) {
   PwDesc& W = *out;
   memset(&W, 0, sizeof(W));
@@ -3143,7 +3254,7 @@ static cudaError_t make_pw(const TcState* S, const adr_plan_s* P, float* u, floa
   W.ind = S->ind;
   W.ind_ctr = S->ind_ctr;
   W.ind_k = kIndSlots;
-  const PwGeom g = pw_geom(S, S->num_sms, share);
+  const PwGeom g = pw_geom(S, S->num_sms, share, ring);
   W.nx = g.nx;
   W.ny = g.ny;
   W.nz = g.nz;
@@ -3154,21 +3265,223 @@ static cudaError_t make_pw(const TcState* S, const adr_plan_s* P, float* u, floa
   W.sy = g.sy;
   W.sz = g.sz;
   if (S->d == 3) {
-    cudaError_t e = encode_field(&W.tu, u, g);
-    if (e == cudaSuccess) e = encode_field(&W.tv, v, g);
+    cudaError_t e = encode_field(&W.tu, u, g, ring);
+    if (e == cudaSuccess) e = encode_field(&W.tv, v, g, ring);
     return e;
   }
   return cudaSuccess;
 }
 
-static int rhs_blocks_of(const TcState* S, double share = 1.0) {
-  const PwGeom g = pw_geom(S, S->num_sms, share);
+static int rhs_blocks_of(const TcState* S, bool ring, double share = 1.0) {
+  const PwGeom g = pw_geom(S, S->num_sms, share, ring);
   if (S->d == 3) return g.xsegs * g.ytiles * g.zsegs;
   const int64_t warps = (int64_t)g.xsegs * g.zsegs;
   return (int)((warps + kPwWarps - 1) / kPwWarps);
 }
 static int rdiff_blocks_of(const TcState* S) {
   return (int)((S->N + kFlatPerBlock - 1) / kFlatPerBlock);
+}
+
+// ---------------------------------------------------------------- two-pass launches, host side
+// Tiling of one product.  kg: how many 128-row groups of Phi share one
+// contraction range (fixed per plan, so that results do not depend on the
+// tile width); bn: the tile width.
+struct TpGeo {
+  int M, N, K, R, tiles_m, tn, bn, kg;
+};
+// Clocks of one K16 step on an N-wide tile: six MMAs, 99 clocks each up to
+// N = 128 and about N / 2 beyond.
+static double tp_step_clk(int bn) { return 6.0 * std::max(99, bn / 2 + 4); }
+// K blocks [k0, k1) of kg 128-row groups of Phi from g0: the union of their
+// column supports.
+static void tp_k_range(const TcState* S, int c, int mu, int ell, int g0, int kg, int& k0, int& k1) {
+  const int n = (int)S->n[mu], ng = (n + 127) / 128, nk = (n + kTpBK - 1) / kTpBK;
+  int lo = n, hi = 0;
+  for (int g = g0; g < std::min(ng, g0 + kg) && S->ksupport; ++g) {
+    const int2 r = S->hband[c][mu][ell][g];
+    if (r.x < r.y) {
+      lo = std::min(lo, r.x);
+      hi = std::max(hi, r.y);
+    }
+  }
+  k0 = lo < hi ? lo / kTpBK : 0;
+  k1 = lo < hi ? std::min(nk, (hi + kTpBK - 1) / kTpBK) : nk;
+}
+// K blocks summed over the components and the groups of kg row groups.
+static double tp_k_sum(const TcState* S, int mu, int ell, int kg) {
+  const int ng = (int)((S->n[mu] + 127) / 128);
+  double sum = 0;
+  for (int c = 0; c < 2; ++c)
+    for (int g0 = 0; g0 < ng; g0 += kg) {
+      int k0, k1;
+      tp_k_range(S, c, mu, ell, g0, kg, k0, k1);
+      sum += k1 - k0;
+    }
+  return sum;
+}
+// share: the solve's part of its launch's points (1 alone).  A narrower tile
+// re-reads the rows but spreads a small grid over more SMs: the width whose
+// waves x time is least is taken, by the clocks above.
+static TpGeo tp_geo(const TcState* S, int mu, int ell, double share) {
+  TpGeo g;
+  g.N = g.K = (int)S->n[mu];
+  g.M = (int)(S->N / g.N);
+  g.R = S->d == 2 ? g.M : (mu == 0 ? (int)S->n[1] : (mu == 1 ? (int)S->n[0] : g.M));
+  g.tiles_m = (g.M + kBM - 1) / kBM;
+  // up to 256 points the groups share one range and can share one tile;
+  // longer rows run 128-row groups (narrower ranges) or 256-row ones (wider
+  // tiles), whichever is less work
+  int width;
+  if (g.N <= 256) {
+    g.kg = (g.N + 127) / 128;
+    width = (g.N + 15) / 16 * 16;
+  } else {
+    g.kg = tp_k_sum(S, mu, ell, 1) * tp_step_clk(128) <= tp_k_sum(S, mu, ell, 2) * tp_step_clk(256) ? 1 : 2;
+    width = 128 * g.kg;
+  }
+  const int ng = (g.N + 128 * g.kg - 1) / (128 * g.kg);
+  const double kavg = (kTpBK / 16) * tp_k_sum(S, mu, ell, g.kg) / (2.0 * ng);  // K16 steps a tile
+  double best = 0;
+  for (int split = 1; split <= 8; split *= 2) {
+    const int bn = ((width + split - 1) / split + 15) / 16 * 16;
+    if (split > 1 && bn < 32) break;
+    const int tn = (g.N + bn - 1) / bn;
+    const double waves = std::max(1.0, std::ceil(2.0 * g.tiles_m * tn / share / S->num_sms));
+    const double t = waves * kavg * tp_step_clk(bn) + 8.0 * bn;
+    if (best == 0 || t < 0.97 * best) {
+      best = t;
+      g.bn = bn;
+      g.tn = tn;
+    }
+  }
+  return g;
+}
+static int tp_slabs(const TcState* S) { return S->d == 3 ? (int)S->n[2] : 1; }
+// Dependency counters of the two-pass launch at the narrowest tiles.
+static int64_t tp_dep_words_max(const TcState* S) {
+  return 2 * (int64_t)tp_slabs(S) * ((S->n[0] + 31) / 32 + 8);
+}
+static int tp_npass(const TcPass& ps) { return ps.fused ? 2 : 1; }
+
+// The descriptors of one launch (dep: this solve's counters).
+static cudaError_t make_tp(const TcState* S, const adr_plan_s* P, const TcPass& ps, float* u, float* v,
+                           double share, uint32_t* dep, TpOp* out) {
+  memset(out, 0, sizeof(*out));
+  float* stage[2] = {(float*)P->u2, (float*)P->v2};
+  float* state[2] = {u, v};
+  const double tau = P->prob.tau;
+  TpGeo geo0{};
+  for (int k = 0; k < tp_npass(ps); ++k) {
+    TpPass& D = out->p[k];
+    const int mu = ps.fused ? k : 2;
+    const TpGeo g = tp_geo(S, mu, ps.ell, share);
+    if (k == 0) geo0 = g;
+    const bool last = !ps.fused || (k == 1 && S->d == 2);
+    D.M = g.M;
+    D.N = g.N;
+    D.K = g.K;
+    D.R = g.R;
+    D.tiles_m = g.tiles_m;
+    D.tn = g.tn;
+    D.bn = g.bn;
+    D.kg_log2 = g.kg == 2;
+    D.per_mul = (uint32_t)((1ull << 32) / (2 * g.tn) + 1);
+    D.slabs = tp_slabs(S);
+    D.dep = ps.fused ? dep : nullptr;
+    D.dep_tn = D.slabs > 1 ? 1 : geo0.tn;
+    D.dep_want = D.slabs > 1 ? geo0.tn : 1;
+    D.dep_r = geo0.R;
+    D.alpha = ps.alpha == kAlphaTau ? (float)tau
+                                    : (ps.alpha == kAlphaTauD ? (float)ldexp(tau, S->d - 1) : 1.0f);
+    for (int c = 0; c < 2; ++c) {
+      const __nv_bfloat16* in = mu == 2 ? S->mid[c] : S->buf[k][c];
+      cudaError_t e = mu == 2 ? encode_pieces_mn(&D.amap[c], in, g.M, g.K, kTpBK)
+                              : encode_tp(&D.amap[c], in, g.K, g.M, kBM, kPieces);
+      if (e == cudaSuccess) e = encode_tp(&D.bmap[c], S->phi[c][mu][ps.ell], g.K, g.N, g.bn, 1);
+      if (e == cudaSuccess) e = encode_tp(&D.bmap[2 + c], S->phi[c][mu][ps.ell], g.K, g.N, g.bn > 128 ? 256 : 128, kPieces);
+      if (e != cudaSuccess) return e;
+      const int ng = (g.N + 127) / 128, nk = (g.K + kTpBK - 1) / kTpBK;
+      for (int q = 0; q * g.kg < ng; ++q) {
+        int k0, k1;
+        tp_k_range(S, c, mu, ps.ell, q * g.kg, g.kg, k0, k1);
+        D.kb[c][q][0] = (uint8_t)k0;
+        D.kb[c][q][1] = (uint8_t)std::min(nk, k1);
+      }
+      if (!last) {
+        D.outp[c] = k == 0 ? S->buf[1][c] : S->mid[c];
+        continue;
+      }
+      D.outf[c] = ps.out == kOutStage ? stage[c] : state[c];
+      D.base[c] = ps.base == kBaseStage ? stage[c] : (ps.base == kBaseState ? state[c] : nullptr);
+      D.lo[c] = S->comp ? S->lo[c] : nullptr;
+    }
+    if (last && S->ind && S->scheme == ADR_ETD2RKDS && ps.out == kOutState) {
+      D.ind = S->ind;
+      D.ind_ctr = S->ind_ctr;
+      D.ind_k = kIndSlots;
+      D.ind_n1 = (int)S->n[0];
+      D.ind_n2 = S->d == 3 ? (int)S->n[1] : 0;
+    }
+  }
+  return cudaSuccess;
+}
+// Units of pass k of a launch.
+static int tp_units(const TcState* S, const TcPass& ps, int k, double share) {
+  const TpGeo g = tp_geo(S, ps.fused ? k : 2, ps.ell, share);
+  return 2 * g.tiles_m * g.tn;
+}
+static int tp_max_bn(const TcState* S, const TcPass& ps, double share) {
+  int b = 0;
+  for (int k = 0; k < tp_npass(ps); ++k) b = std::max(b, tp_geo(S, ps.fused ? k : 2, ps.ell, share).bn);
+  return b;
+}
+static int tp_dep_words(const TcState* S, const TcPass& ps, double share) {
+  return ps.fused ? 2 * tp_slabs(S) * tp_geo(S, 0, ps.ell, share).tn : 0;
+}
+// Order of a two-pass launch's units.  Both passes run slab by slab, so on a
+// large 3D grid the x2 tiles of a run of slabs follow the x1 tiles of the
+// next run: the pieces between the passes are then read from L2 (201 MB at
+// 256^3 would not stay there).  chunks = 1: all of pass 0, then all of pass 1.
+static int tp_chunks(const TcState* S, const TcPass& ps, int sms) {
+  if (!ps.fused || S->d != 3 || 12.0 * (double)S->N < 64e6) return 1;
+  const TpGeo g0 = tp_geo(S, 0, ps.ell, 1.0), g1 = tp_geo(S, 1, ps.ell, 1.0);
+  const int64_t u0 = 2 * (int64_t)g0.tiles_m * g0.tn, u1 = 2 * (int64_t)g1.tiles_m * g1.tn;
+  for (int c = 8; c > 1; --c) {
+    if (u0 / c < 2 * sms) continue;
+    bool ok = true;  // pass 1's chunk i reads nothing beyond pass 0's chunk i + 1
+    for (int i = 0; i + 1 < c && ok; ++i) {
+      const int64_t mt1 = ((i + 1) * u1 / c - 1) / (2 * g1.tn);
+      const int64_t row1 = std::min<int64_t>((mt1 + 1) * kBM, g1.M) - 1;
+      const int64_t need = (((row1 / g1.R + 1) * g0.R - 1) / kBM + 1) * 2 * g0.tn;
+      ok = need <= (i + 2) * u0 / c;
+    }
+    if (ok) return c;
+  }
+  return 1;
+}
+static void tp_sequence(TpLaunch& L, int npass, const int nu[2], int chunks) {
+  L.npass = npass;
+  L.nunits = nu[0] + (npass > 1 ? nu[1] : 0);
+  int end = 0, k = 0;
+  auto add = [&](int pass, int i) {
+    const int a = (int)((int64_t)i * nu[pass] / chunks), b = (int)((int64_t)(i + 1) * nu[pass] / chunks);
+    end += b - a;
+    L.seq_end[k] = end;
+    L.seq_first[k] = a;
+    L.seq_pass[k] = pass;
+    ++k;
+  };
+  if (npass == 1) {
+    chunks = 1;
+    add(0, 0);
+  } else {
+    add(0, 0);
+    for (int i = 0; i < chunks; ++i) {
+      if (i + 1 < chunks) add(0, i + 1);
+      add(1, i);
+    }
+  }
+  L.nseq = k;
 }
 
 void tc_init(TcOperands* t) { memset(t, 0, sizeof(*t)); }
@@ -3181,6 +3494,35 @@ void tc_free(TcOperands* t) {
     delete S;
   }
   t->work[0] = nullptr;
+}
+
+// Whether the first two directions run as the two-pass launch (tp_kernel)
+// rather than with the intermediate in TMEM (tc_fused_kernel).  us a step,
+// tc_fused_kernel / tp_kernel, plain ETD2RKds:
+//   2D  n2 <= 256, up to 32768 points (64^2 19.2 / 23.6, 128^2 25.8 / 30.4):
+//       TMEM, one launch's latency; beyond that (Brusselator 200^2 49.5 / 40.8,
+//       256^2 52.5 / 39.2) two passes: a unit of tc_fused_kernel holds all of
+//       x2, and a row of tiles is one SM's work;
+//   2D  n2 > 256 and some x2 tile's support wider than the 256 intermediate
+//       columns (384^2 65.5 / 46.7, 512^2 77.0 / 53.9, 1024^2 167 / 86): the
+//       intermediate is computed again for every tile it reaches;
+//       narrower supports (FHN 384^2 40.0 / 40.5, 1024^2 46.0 / 54.0): TMEM;
+//   3D  up to 10^7 points (128^3 104 / 98, 160^3 281 / 188, 192^3 382 / 295),
+//       and above where 128-row tiles pad the slabs by over 10%: two passes;
+//       256^3 (691 / 720): TMEM, whose intermediate saves HBM traffic.
+static bool tp_better(const TcState* S) {
+  const int64_t n1 = S->n[0], n2 = S->n[1];
+  if (S->d == 3) {
+    auto up = [](int64_t n) { return (double)((n + kBM - 1) / kBM * kBM); };
+    return S->N <= 10000000 || up(n1) * up(n2) > 1.1 * (double)(n1 * n2);
+  }
+  if (n2 <= kFRowsW) return n1 * n2 > 32768;
+  if (!S->ksupport) return true;
+  for (int c = 0; c < 2; ++c)
+    for (int l = 0; l < 3; ++l)
+      for (const int2& r : S->hband[c][1][l])
+        if (r.y - r.x > kFRowsW) return true;
+  return false;
 }
 
 cudaError_t tc_prepare(TcOperands* t, int prec, int scheme, int d, const int64_t n[3],
@@ -3197,6 +3539,7 @@ cudaError_t tc_prepare(TcOperands* t, int prec, int scheme, int d, const int64_t
     if ((e = set_smem_attr<64, 64>()) != cudaSuccess) return e;
     if ((e = set_smem_attr_pair<64>()) != cudaSuccess) return e;
     if ((e = set_smem_attr_pair<128>()) != cudaSuccess) return e;
+    if ((e = set_tp_attr()) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(tc_fused_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                   kFSmem)) != cudaSuccess)
       return e;
@@ -3335,6 +3678,21 @@ cudaError_t tc_prepare(TcOperands* t, int prec, int scheme, int d, const int64_t
                           kVariants[S->variant].cta2 ? bn / 2 : bn, sw, S->fmt);
         if (e != cudaSuccess) return e;
       }
+  // host copies of the supports, ordered on the plan's stream (a copy on the
+  // legacy stream would wait for every other stream's queued work)
+  for (int c = 0; c < 2; ++c)
+    for (int m = 0; m < d; ++m)
+      for (int l = 0; l < 3; ++l)
+        if (!S->hband[c][m][l].empty()) {
+          e = cudaMemcpyAsync(S->hband[c][m][l].data(), S->kband[c][m][l],
+                              sizeof(int2) * S->hband[c][m][l].size(), cudaMemcpyDeviceToHost, s);
+          if (e != cudaSuccess) return e;
+        }
+  e = cudaStreamSynchronize(s);  // the split matrices and the supports' copies are complete
+  if (e != cudaSuccess) return e;
+  // no kernel requested: the library's own choice
+  S->tp = S->fused12 && variant_req < 0 && getenv("ADR_TC_VARIANT") == nullptr && tp_better(S);
+  if (S->tp) S->variant = 0;  // one step sequence for every grid: all group in a batch
   S->lo[0] = S->lo[1] = nullptr;
   S->comp_u = S->comp_v = nullptr;
   S->ind = nullptr;
@@ -3355,7 +3713,14 @@ cudaError_t tc_prepare(TcOperands* t, int prec, int scheme, int d, const int64_t
         if (e != cudaSuccess) return e;
       }
     }
-  if (S->fused12) {
+  if (S->tp) {
+    for (int c = 0; c < 2 && d == 3; ++c)
+      if ((e = alloc((void**)&S->mid[c], (size_t)kPieces * 2 * S->N)) != cudaSuccess) return e;
+    const size_t words = 4 * (2 + (size_t)tp_dep_words_max(S));
+    if ((e = alloc((void**)&S->tpctl, words)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(S->tpctl, 0, words, s)) != cudaSuccess) return e;
+  }
+  if (S->fused12 && !S->tp) {
     for (int c = 0; c < 2; ++c) {
       for (int l = 0; l < 3; ++l) {
         if (!S->phi[c][0][l]) continue;
@@ -3378,13 +3743,13 @@ cudaError_t tc_prepare(TcOperands* t, int prec, int scheme, int d, const int64_t
     int b = 0;
     if (S->fused12) {  // reads buffer 0; 2D: writes the operator's result
       if (d == 3) {    // modes 1 and 2 to pieces in buffer 1, then mode 3 from them
-        TcPass f{0, 0, ell, kPieces3, 0, kOutPieces, kBaseNone, kAlphaOne, 1, 0};
+        TcPass f{0, 0, ell, kPieces3, 0, kOutPieces, kBaseNone, kAlphaOne, 1, 0, S->tp};
         S->passes.push_back(f);
         S->ops.push_back({kOpTc, (int)S->passes.size() - 1, 0.f});
-        TcPass m3{1, 2, ell, kAxpy, 0, last_out, last_base, last_alpha, 0, 1};
+        TcPass m3{1, 2, ell, kAxpy, 0, last_out, last_base, last_alpha, 0, 1, S->tp};
         S->passes.push_back(m3);
       } else {
-        TcPass f{0, 0, ell, kAxpy, 0, last_out, last_base, last_alpha, 1, 0};
+        TcPass f{0, 0, ell, kAxpy, 0, last_out, last_base, last_alpha, 1, 0, S->tp};
         S->passes.push_back(f);
       }
       S->ops.push_back({kOpTc, (int)S->passes.size() - 1, 0.f});
@@ -3423,13 +3788,13 @@ cudaError_t tc_prepare(TcOperands* t, int prec, int scheme, int d, const int64_t
     const int b2 = S->fuse ? b1 : 0;
     if (S->fused12) {
       if (d == 3) {
-        TcPass f{b2, 0, 2, kPieces3, 0, kOutPieces, kBaseNone, kAlphaOne, 1, 0};
+        TcPass f{b2, 0, 2, kPieces3, 0, kOutPieces, kBaseNone, kAlphaOne, 1, 0, S->tp};
         S->passes.push_back(f);
         S->ops.push_back({kOpTc, (int)S->passes.size() - 1, 0.f});
-        TcPass m3{1 - b2, 2, 2, kAxpy, 0, kOutState, kBaseStage, kAlphaTauD, 0, 1};
+        TcPass m3{1 - b2, 2, 2, kAxpy, 0, kOutState, kBaseStage, kAlphaTauD, 0, 1, S->tp};
         S->passes.push_back(m3);
       } else {
-        TcPass f{b2, 0, 2, kAxpy, 0, kOutState, kBaseStage, kAlphaTauD, 1, 0};
+        TcPass f{b2, 0, 2, kAxpy, 0, kOutState, kBaseStage, kAlphaTauD, 1, 0, S->tp};
         S->passes.push_back(f);
       }
       S->ops.push_back({kOpTc, (int)S->passes.size() - 1, 0.f});
@@ -3447,20 +3812,10 @@ cudaError_t tc_prepare(TcOperands* t, int prec, int scheme, int d, const int64_t
     }
   }
   const int np = (int)S->passes.size();
-  for (int p = 0; p < np; ++p) S->units[p] = units_of(S, S->passes[p], bn);
-  S->rhs_blocks = rhs_blocks_of(S);
+  for (int p = 0; p < np && !S->tp; ++p) S->units[p] = units_of(S, S->passes[p], bn);
+  S->rhs_blocks = rhs_blocks_of(S, row_ring(S));
   S->rdiff_blocks = rdiff_blocks_of(S);
-  // host copies of the supports, ordered on the plan's stream (a copy on the
-  // legacy stream would wait for every other stream's queued work)
-  for (int c = 0; c < 2; ++c)
-    for (int m = 0; m < d; ++m)
-      for (int l = 0; l < 3; ++l)
-        if (!S->hband[c][m][l].empty()) {
-          e = cudaMemcpyAsync(S->hband[c][m][l].data(), S->kband[c][m][l],
-                              sizeof(int2) * S->hband[c][m][l].size(), cudaMemcpyDeviceToHost, s);
-          if (e != cudaSuccess) return e;
-        }
-  e = cudaStreamSynchronize(s);  // the split matrices and the supports' copies are complete
+  e = cudaStreamSynchronize(s);  // the buffers are cleared
   if (e != cudaSuccess) return e;
   S->bound_u = S->bound_v = nullptr;
   t->ready = 1;
@@ -3506,9 +3861,17 @@ cudaError_t tc_bind(TcOperands* t, adr_plan_s* P, void* u, void* v) {
   if (!S || !t->ready) return cudaErrorNotSupported;
   if (S->bound_u == u && S->bound_v == v) return cudaSuccess;
   const int np = (int)S->passes.size();
-  S->h_desc.resize(np);
-  for (int p = 0; p < np; ++p) S->h_desc[p] = make_desc(S, P, S->passes[p], (float*)u, (float*)v);
-  cudaError_t e = make_pw(S, P, (float*)u, (float*)v, &S->h_pw);
+  cudaError_t e = cudaSuccess;
+  if (S->tp) {
+    S->h_op.resize(np);
+    for (int p = 0; p < np && e == cudaSuccess; ++p)
+      e = make_tp(S, P, S->passes[p], (float*)u, (float*)v, 1.0, S->tpctl + 2, &S->h_op[p]);
+    if (e != cudaSuccess) return e;
+  } else {
+    S->h_desc.resize(np);
+    for (int p = 0; p < np; ++p) S->h_desc[p] = make_desc(S, P, S->passes[p], (float*)u, (float*)v);
+  }
+  e = make_pw(S, P, (float*)u, (float*)v, &S->h_pw, row_ring(S));
   if (e != cudaSuccess) return e;
   S->bound_u = u;
   S->bound_v = v;
@@ -3533,6 +3896,15 @@ struct GroupStep {
   int ind[16];              // per pass: accumulates the step's indicators
   int df;                   // reactions in double-float (ADR_STATE_COMPENSATED)
   int xslots;               // resident clusters of the exchanging kernel
+  // two-pass launches
+  int tp;
+  const TpOp* hop;          // one solve: host copies [np]; else null
+  const TpOp* dop;          // [np][nsolves]
+  const int* tpus;          // [np][2][nsolves + 1]
+  int tpnu[16][2], tpbn[16], tpchunks[16], tpnctl[16];
+  uint32_t* tpctl;
+  int tpclear;              // no pointwise kernel between the operator launches
+  int ring, nseg;           // 3D stencil on whole rows, 64-point segments of the widest
   PwLaunch rhs, flat;       // stencil blocks; flat pointwise blocks
   int rhs_blocks, flat_blocks;
   int* err;
@@ -3543,14 +3915,45 @@ struct GroupStep {
 static cudaError_t group_step(adr_plan_s* ctl, const GroupStep& G) {
   const double N = G.pw_n;
   cudaStream_t st = ctl->stream;
+  // a pointwise kernel that writes an operator's input clears the claims of
+  // the two-pass launch that follows it
+  auto opens = [&](const PwLaunch& L) {
+    PwLaunch R = L;
+    R.err = G.err;
+    if (G.tp) {
+      R.ctl = G.tpctl;
+      for (int p = 0; p < G.np; ++p) R.nctl = std::max(R.nctl, G.tpnctl[p]);
+    }
+    return R;
+  };
   for (int o = 0; o < G.nops; ++o) {
     const TcOp& op = G.ops[o];
     cudaError_t e = cudaSuccess;
+    if (G.tp && op.kind == kOpTc) {
+      const int p = op.pass;
+      TpLaunch L;
+      memset(&L, 0, sizeof(L));
+      if (G.hop) {
+        L.one = G.hop[p];
+      } else {
+        L.desc = G.dop + (size_t)p * G.nsolves;
+        L.ustart = G.tpus + (size_t)p * 2 * (G.nsolves + 1);
+      }
+      L.nsolves = G.nsolves;
+      tp_sequence(L, G.fused[p] ? 2 : 1, G.tpnu[p], G.tpchunks[p]);
+      L.ctl = G.tpctl;
+      L.nctl = G.tpnctl[p];
+      L.clear = G.tpclear;
+      L.err = G.err;
+      e = timed_kernel(ctl, KC_MODE_TC, G.flops[p], G.bytes[p],
+                       [&] { return launch_tp(G.fslots, st, L, !G.fused[p], G.tpbn[p], G.ind[p] ? 2 : (G.df ? 1 : 0)); });
+      if (e != cudaSuccess) return e;
+      continue;
+    }
     switch (op.kind) {
       case kOpRhs:
         e = timed_kernel(ctl, KC_RHS, N * 2.0 * (6.0 * G.d + 10.0), N * (8.0 + 12.0), [&] {
-          PwLaunch R = G.rhs;
-          R.err = G.err;
+          const PwLaunch R = opens(G.rhs);
           const dim3 gr(G.rhs_blocks), bl(kPwThreads);
           if (G.fmt == kFmtTF32) {
             if (G.d == 3)
@@ -3559,6 +3962,9 @@ static cudaError_t group_step(adr_plan_s* ctl, const GroupStep& G) {
             return G.df ? launch_k(rhs_pieces_kernel<kZB2, kFmtTF32, true>, gr, bl, 0, st, R)
                         : launch_k(rhs_pieces_kernel<kZB2, kFmtTF32>, gr, bl, 0, st, R);
           }
+          if (G.d == 3 && G.ring)
+            return G.df ? launch_rhs3_rows<true>(G.nseg, G.rhs_blocks, st, R)
+                        : launch_rhs3_rows<false>(G.nseg, G.rhs_blocks, st, R);
           if (G.d == 3)
             return G.df ? launch_k(rhs3_ring_kernel<kFmtBF16, true>, gr, bl, kRingSmem, st, R)
                         : launch_k(rhs3_ring_kernel<>, gr, bl, kRingSmem, st, R);
@@ -3571,7 +3977,7 @@ static cudaError_t group_step(adr_plan_s* ctl, const GroupStep& G) {
           const dim3 gr(G.flat_blocks), bl(kPwThreads);
           if (G.fmt == kFmtTF32)
             return launch_k(rdiff_pieces_kernel<kFmtTF32>, gr, bl, 0, st, G.flat);
-          return launch_k(rdiff_pieces_kernel<>, gr, bl, 0, st, G.flat);
+          return launch_k(rdiff_pieces_kernel<>, gr, bl, 0, st, opens(G.flat));
         });
         break;
       case kOpLawsonPre:
@@ -3580,7 +3986,7 @@ static cudaError_t group_step(adr_plan_s* ctl, const GroupStep& G) {
             return launch_k(lawson_pre_pieces_kernel<kFmtTF32>, dim3(G.flat_blocks), dim3(kPwThreads),
                             0, st, G.flat, op.factor);
           return launch_k(lawson_pre_pieces_kernel<>, dim3(G.flat_blocks), dim3(kPwThreads), 0, st,
-                          G.flat, op.factor);
+                          opens(G.flat), op.factor);
         });
         break;
       case kOpLawsonPost:
@@ -3652,6 +4058,23 @@ static void fill_ops(GroupStep& G, const TcState* S) {
   G.fslots = S->num_sms;
   G.fmt = S->fmt;
   G.df = S->comp == 2;
+  G.tp = S->tp;
+  G.ring = row_ring(S);
+  G.nseg = (int)((S->n[0] + 63) / 64);
+}
+// The two-pass launches of a plan on its own.
+static void fill_tp_one(GroupStep& G, const TcState* S) {
+  G.hop = S->h_op.data();
+  G.tpctl = S->tpctl;
+  for (int p = 0; p < G.np; ++p) {
+    const TcPass& ps = S->passes[p];
+    for (int k = 0; k < tp_npass(ps); ++k) G.tpnu[p][k] = tp_units(S, ps, k, 1.0);
+    G.tpbn[p] = tp_max_bn(S, ps, 1.0);
+    G.tpchunks[p] = tp_chunks(S, ps, S->num_sms);
+    G.tpnctl[p] = 2 + tp_dep_words(S, ps, 1.0);
+    G.ind[p] = S->h_op[p].p[0].ind != nullptr || S->h_op[p].p[1].ind != nullptr;
+    pass_work(S, ps, G.flops[p], G.bytes[p]);
+  }
 }
 
 cudaError_t tc_step(TcOperands* t, adr_plan_s* P, void* u, void* v) {
@@ -3667,7 +4090,8 @@ cudaError_t tc_step(TcOperands* t, adr_plan_s* P, void* u, void* v) {
   G.desc = nullptr;
   G.hdesc = S->h_desc.data();
   G.ustart = nullptr;
-  for (int p = 0; p < G.np; ++p) {
+  if (S->tp) fill_tp_one(G, S);
+  for (int p = 0; p < G.np && !S->tp; ++p) {
     G.units[p] = S->units[p];
     G.ind[p] = S->h_desc[p].ind != nullptr;
     pass_work(S, S->passes[p], G.flops[p], G.bytes[p]);
@@ -3710,6 +4134,22 @@ void tc_mode_macs(const TcOperands* t, double* dense, double* computed) {
   const int bk = kVariants[S->variant].sw / (S->fmt == kFmtTF32 ? 4 : 2);
   static const std::vector<int2> none;
   for (const TcPass& ps : S->passes) {
+    if (ps.tp) {  // per 128-row tile: the contraction range of its group, clipped to n
+      for (int k = 0; k < tp_npass(ps); ++k) {
+        const int mu = ps.fused ? k : 2;
+        const TpGeo g = tp_geo(S, mu, ps.ell, 1.0);
+        for (int c = 0; c < 2; ++c) {
+          *dense += (double)g.M * g.N * g.K;
+          for (int g0 = 0; g0 * 128 < g.N; g0 += g.kg) {
+            int k0, k1;
+            tp_k_range(S, c, mu, ps.ell, g0, g.kg, k0, k1);
+            *computed += (double)g.M * std::min(128 * g.kg, g.N - g0 * 128) *
+                         (std::min(g.K, k1 * kTpBK) - k0 * kTpBK);
+          }
+        }
+      }
+      continue;
+    }
     if (ps.fused) {  // both products of tc_fused_kernel, as its loops run them
       const int64_t n1 = S->n[0], n2 = S->n[1], slabs = S->N / (n1 * n2);
       const int64_t tn = (n2 + kBM - 1) / kBM, bunit = n2 <= kFRowsW ? tn : 1;
@@ -3789,7 +4229,9 @@ cudaError_t tc_time_passes(TcOperands* t, adr_plan_s* P, void* u, void* v, int r
   G.nops = k;
   *passes = k;
   G.hdesc = S->h_desc.data();
-  for (int p = 0; p < G.np; ++p) {
+  if (S->tp) fill_tp_one(G, S);
+  G.tpclear = 1;  // the launches follow one another without row kernels between
+  for (int p = 0; p < G.np && !S->tp; ++p) {
     G.units[p] = S->units[p];
     G.ind[p] = S->h_desc[p].ind != nullptr;
     pass_work(S, S->passes[p], G.flops[p], G.bytes[p]);
@@ -3818,6 +4260,9 @@ cudaError_t tc_time_passes(TcOperands* t, adr_plan_s* P, void* u, void* v, int r
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (e == cudaSuccess) e = cudaEventCreate(&e0);
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
+  // no row kernel clears the claims before the first launch
+  if (e == cudaSuccess && S->tp)
+    e = cudaMemsetAsync(S->tpctl, 0, 4 * (2 + (size_t)tp_dep_words_max(S)), P->stream);
   if (e == cudaSuccess) e = cudaGraphLaunch(ge, P->stream);
   if (e == cudaSuccess) e = cudaEventRecord(e0, P->stream);
   if (e == cudaSuccess) e = cudaGraphLaunch(ge, P->stream);
@@ -3916,6 +4361,13 @@ struct adr_batch_s {
   int units[8];
   int rhs_blocks, rdiff_blocks;
   double flops[8], bytes[8], pw_n;
+  // two-pass launches
+  TpOp* d_op;           // [np][nsolves]
+  int* d_tpus;          // [np][2][nsolves + 1]
+  uint32_t* d_tpctl;
+  std::vector<std::vector<int>> dep_at;   // [np][nsolves]: offset of a solve's counters
+  int tpnu[8][2], tpbn[8], tpnctl[8];
+  int ring, nseg;       // 3D stencil: whole rows if every solve's fit, segments of the widest
   std::vector<void*> bound_u, bound_v;
   int ind_pass[8];      // per pass: some solve of the binding has indicators on
   // CUDA graph of kBatchChunk steps
@@ -4139,6 +4591,41 @@ static adr_status batch_create_any(const adr_plan* plans, int count, void* strea
   return ADR_OK;
 }
 
+// Tables of a grouped batch of two-pass launches: units per pass, claims and
+// dependency counters (sizes depend on the solves alone).
+template <typename Alloc>
+static cudaError_t batch_create_tp(adr_batch B, cudaStream_t stream, Alloc& alloc) {
+  const int S_ = B->nsolves;
+  std::vector<int> us((size_t)B->np * 2 * (S_ + 1));
+  auto state = [&](int i) { return (const TcState*)B->plans[i]->tc.work[0]; };
+  int words = 0;
+  B->dep_at.assign(B->np, std::vector<int>(S_));
+  for (int p = 0; p < B->np; ++p) {
+    int acc[2] = {0, 0}, dep = 0;
+    for (int i = 0; i < S_; ++i) {
+      const TcState* S = state(i);
+      const double share = (double)S->N / B->pw_n;
+      const TcPass& ps = S->passes[p];
+      for (int k = 0; k < 2; ++k) {
+        us[((size_t)p * 2 + k) * (S_ + 1) + i] = acc[k];
+        if (k < tp_npass(ps)) acc[k] += tp_units(S, ps, k, share);
+      }
+      B->tpbn[p] = std::max(i ? B->tpbn[p] : 0, tp_max_bn(S, ps, share));
+      B->dep_at[p][i] = 2 + dep;
+      dep += tp_dep_words(S, ps, share);
+    }
+    for (int k = 0; k < 2; ++k) us[((size_t)p * 2 + k) * (S_ + 1) + S_] = B->tpnu[p][k] = acc[k];
+    B->tpnctl[p] = 2 + dep;
+    words = std::max(words, 2 + dep);
+  }
+  cudaError_t e = alloc((void**)&B->d_op, sizeof(TpOp) * B->np * S_);
+  if (e == cudaSuccess) e = alloc((void**)&B->d_tpus, sizeof(int) * us.size());
+  if (e == cudaSuccess) e = alloc((void**)&B->d_tpctl, sizeof(uint32_t) * words);
+  if (e == cudaSuccess) e = g_upload_ring.upload(B->d_tpus, us.data(), sizeof(int) * us.size(), stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(B->d_tpctl, 0, sizeof(uint32_t) * words, stream);
+  return e;
+}
+
 static adr_status batch_create_one(const adr_plan* plans, int count, void* stream, adr_batch* out) {
   adr_batch B = new adr_batch_s();
   B->plans.assign(plans, plans + count);
@@ -4185,7 +4672,7 @@ static adr_status batch_create_one(const adr_plan* plans, int count, void* strea
       for (int i = 0; i < S_; ++i) {
         const TcState* S = (const TcState*)plans[i]->tc.work[0];
         us[(size_t)p * (S_ + 1) + i] = acc;
-        acc += units_of(S, S->passes[p], bn);
+        acc += S->tp ? 0 : units_of(S, S->passes[p], bn);
         double f, b;
         pass_work(S, S->passes[p], f, b);
         B->flops[p] += f;
@@ -4195,12 +4682,19 @@ static adr_status batch_create_one(const adr_plan* plans, int count, void* strea
       B->units[p] = acc;
     }
     int ra = 0, rd = 0;
-    for (int i = 0; i < S_; ++i) B->pw_n += (double)((const TcState*)plans[i]->tc.work[0])->N;
+    B->ring = 1;
+    B->nseg = 1;
+    for (int i = 0; i < S_; ++i) {
+      const TcState* S = (const TcState*)plans[i]->tc.work[0];
+      B->pw_n += (double)S->N;
+      B->ring = B->ring && row_ring(S);
+      B->nseg = std::max(B->nseg, (int)((S->n[0] + 63) / 64));
+    }
     for (int i = 0; i < S_; ++i) {
       const TcState* S = (const TcState*)plans[i]->tc.work[0];
       bs[i] = ra;
       bs[(S_ + 1) + i] = rd;
-      ra += rhs_blocks_of(S, (double)S->N / B->pw_n);
+      ra += rhs_blocks_of(S, B->ring != 0, (double)S->N / B->pw_n);
       rd += rdiff_blocks_of(S);
     }
     bs[S_] = ra;
@@ -4216,6 +4710,7 @@ static adr_status batch_create_one(const adr_plan* plans, int count, void* strea
     if (e == cudaSuccess)
       e = g_upload_ring.upload(B->d_bstart, bs.data(), sizeof(int) * bs.size(), (cudaStream_t)stream);
     if (e == cudaSuccess) e = cudaMemsetAsync(B->d_err, 0, sizeof(int), (cudaStream_t)stream);
+    if (S0->tp && e == cudaSuccess) e = batch_create_tp(B, (cudaStream_t)stream, alloc);
   }
   if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&B->cap, cudaStreamNonBlocking);
   if (e != cudaSuccess) {
@@ -4241,20 +4736,33 @@ static cudaError_t batch_bind(adr_batch B, void* const* u, void* const* v) {
   const int S_ = B->nsolves;
   std::vector<TcPassDesc> hd((size_t)B->np * S_);
   std::vector<PwDesc> hp(S_);
+  const bool tp = B->proto->tp != 0;
+  std::vector<TpOp> hop(tp ? (size_t)B->np * S_ : 0);
   for (int i = 0; i < S_; ++i) {
     adr_plan_s* P = B->plans[i];
     const TcState* S = (const TcState*)P->tc.work[0];
-    for (int p = 0; p < B->np; ++p)
+    for (int p = 0; p < B->np && !S->tp; ++p)
       hd[(size_t)p * S_ + i] = make_desc(S, P, S->passes[p], (float*)u[i], (float*)v[i]);
-    cudaError_t e = make_pw(S, P, (float*)u[i], (float*)v[i], &hp[i], (double)S->N / B->pw_n);
+    if (S->tp) {
+      const double share = (double)S->N / B->pw_n;
+      cudaError_t r = cudaSuccess;
+      for (int p = 0; p < B->np && r == cudaSuccess; ++p)
+        r = make_tp(S, P, S->passes[p], (float*)u[i], (float*)v[i], share, B->d_tpctl + B->dep_at[p][i],
+                    &hop[(size_t)p * S_ + i]);
+      if (r != cudaSuccess) return r;
+    }
+    cudaError_t e = make_pw(S, P, (float*)u[i], (float*)v[i], &hp[i], B->ring != 0, (double)S->N / B->pw_n);
     if (e != cudaSuccess) return e;
   }
   for (int p = 0; p < B->np; ++p) {
     B->ind_pass[p] = 0;
-    for (int i = 0; i < S_; ++i) B->ind_pass[p] |= hd[(size_t)p * S_ + i].ind != nullptr;
+    for (int i = 0; i < S_; ++i)
+      B->ind_pass[p] |= tp ? (hop[(size_t)p * S_ + i].p[0].ind || hop[(size_t)p * S_ + i].p[1].ind)
+                           : hd[(size_t)p * S_ + i].ind != nullptr;
   }
-  cudaError_t e = g_upload_ring.upload(B->d_desc, hd.data(), sizeof(TcPassDesc) * hd.size(),
-                                       B->ctl->stream);
+  cudaError_t e = tp ? g_upload_ring.upload(B->d_op, hop.data(), sizeof(TpOp) * hop.size(), B->ctl->stream)
+                     : g_upload_ring.upload(B->d_desc, hd.data(), sizeof(TcPassDesc) * hd.size(),
+                                            B->ctl->stream);
   if (e == cudaSuccess)
     e = g_upload_ring.upload(B->d_pw, hp.data(), sizeof(PwDesc) * hp.size(), B->ctl->stream);
   if (e != cudaSuccess) return e;
@@ -4286,7 +4794,18 @@ static cudaError_t batch_step_direct(adr_batch B, int64_t nsteps) {
     G.flops[p] = B->flops[p];
     G.bytes[p] = B->bytes[p];
     G.ind[p] = B->ind_pass[p];
+    if (G.tp) {
+      for (int k = 0; k < 2; ++k) G.tpnu[p][k] = B->tpnu[p][k];
+      G.tpbn[p] = B->tpbn[p];
+      G.tpchunks[p] = 1;
+      G.tpnctl[p] = B->tpnctl[p];
+    }
   }
+  G.dop = B->d_op;
+  G.tpus = B->d_tpus;
+  G.tpctl = B->d_tpctl;
+  G.ring = B->ring;
+  G.nseg = B->nseg;
   memset(&G.rhs, 0, sizeof(G.rhs));
   G.rhs.desc = B->d_pw;
   G.rhs.bstart = B->d_bstart;
