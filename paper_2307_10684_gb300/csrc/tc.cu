@@ -3328,17 +3328,12 @@ static TpGeo tp_geo(const TcState* S, int mu, int ell, double share) {
   g.M = (int)(S->N / g.N);
   g.R = S->d == 2 ? g.M : (mu == 0 ? (int)S->n[1] : (mu == 1 ? (int)S->n[0] : g.M));
   g.tiles_m = (g.M + kBM - 1) / kBM;
-  // up to 256 points the groups share one range and can share one tile;
-  // longer rows run 128-row groups (narrower ranges) or 256-row ones (wider
-  // tiles), whichever is less work
-  int width;
-  if (g.N <= 256) {
-    g.kg = (g.N + 127) / 128;
-    width = (g.N + 15) / 16 * 16;
-  } else {
-    g.kg = tp_k_sum(S, mu, ell, 1) * tp_step_clk(128) <= tp_k_sum(S, mu, ell, 2) * tp_step_clk(256) ? 1 : 2;
-    width = 128 * g.kg;
-  }
+  // up to 256 points the 128-row groups share one range, so that tiles of equal
+  // width can split them; longer rows run a range of their own per group
+  // (us a step, one range per 128 / per 256 columns, Brusselator 1024^2
+  // 82.7 / 86.6, 2048 x 1024 153 / 186, FHN 2048 x 1536 132 / 171)
+  g.kg = g.N <= 256 ? (g.N + 127) / 128 : 1;
+  const int width = g.N <= 256 ? (g.N + 15) / 16 * 16 : 128;
   const int ng = (g.N + 128 * g.kg - 1) / (128 * g.kg);
   const double kavg = (kTpBK / 16) * tp_k_sum(S, mu, ell, g.kg) / (2.0 * ng);  // K16 steps a tile
   double best = 0;
@@ -3504,8 +3499,9 @@ void tc_free(TcOperands* t) {
 //       256^2 52.5 / 39.2) two passes: a unit of tc_fused_kernel holds all of
 //       x2, and a row of tiles is one SM's work;
 //   2D  n2 > 256 and some x2 tile's support wider than the 256 intermediate
-//       columns (384^2 65.5 / 46.7, 512^2 77.0 / 53.9, 1024^2 167 / 86): the
-//       intermediate is computed again for every tile it reaches;
+//       columns (384^2 65.7 / 47.1, 512^2 77.0 / 53.1, 1024^2 168 / 83,
+//       FHN 2048 x 1536 160 / 132): the intermediate is computed again for
+//       every tile it reaches;
 //       narrower supports (FHN 384^2 40.0 / 40.5, 1024^2 46.0 / 54.0): TMEM;
 //   3D  up to 10^7 points (128^3 104 / 98, 160^3 281 / 188, 192^3 382 / 295),
 //       and above where 128-row tiles pad the slabs by over 10%: two passes;

@@ -20,9 +20,12 @@
 // per output as in every other kernel here.
 //
 // Tile width.  An MMA takes 99 clocks here whatever its N up to 128, and about
-// N / 2 beyond (measured: 48 ns apart at N = 32, 80 and 128), so the widest
-// tile that fits is the cheapest per output: 160 = one tile, not 2 x 80.
-// Narrower tiles only serve to spread small grids over more SMs (tp_geo).
+// N / 2 beyond (measured: 48 ns apart at N = 32, 80 and 128).  So of tiles that
+// contract over the same range the widest is the cheapest per output: 136^3
+// runs at 145 us a step with one tile of 144 columns, 163 with two of 80
+// (192^3 296 / 312; 160^3 190 / 185, whose epilogues overlap better).  Beyond
+// 256 columns 128-wide tiles with ranges of their own win, and narrower tiles
+// serve to spread small grids over more SMs (tp_geo).
 
 constexpr int kTpBK = 32;                          // K values per stage (64-byte rows)
 constexpr int kTpPieceA = kBM * 64;                // one piece of X's tile
