@@ -17,6 +17,7 @@
 #include <stdint.h>
 #include <string.h>
 
+#include <algorithm>
 #include <string>
 #include <vector>
 
@@ -53,8 +54,9 @@ struct GenPtrs {
 
 // W_c += G_c(U) (stage 1) or W_c = G_c(U2) - G_c(U) (stage 2, u2 set).
 template <typename T>
-__global__ void __launch_bounds__(256) poly_kernel(const __grid_constant__ PolyTerms P, GenPtrs q,
+__global__ void __launch_bounds__(64) poly_kernel(const __grid_constant__ PolyTerms P, GenPtrs q,
                                                    int64_t N, int stage2) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
   for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < N;
        i += (int64_t)gridDim.x * blockDim.x) {
     T u[4] = {(T)0, (T)0, (T)0, (T)0}, g[4];
@@ -69,6 +71,8 @@ __global__ void __launch_bounds__(256) poly_kernel(const __grid_constant__ PolyT
       for (int c = 0; c < P.m; ++c) ((T*)q.w[c])[i] += g[c];
     }
   }
+  // at the end, so that the next kernel's blocks spread over all SMs
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 struct GeneralState {
@@ -85,40 +89,54 @@ struct GeneralState {
   void* t1[4];
 };
 
-static int grid_of(int64_t N) {
-  int64_t b = (N + 255) / 256;
-  if (b > 152 * 16) b = 152 * 16;
-  return (int)(b < 1 ? 1 : b);
+// Blocks of 64: a few thousand points then cover all SMs, whose FP64 rate
+// bounds the polynomials.
+constexpr int kPolyThreads = 64;
+template <typename T>
+static cudaError_t launch_poly(const PolyTerms& terms, const GenPtrs& q, int64_t N, int stage2, cudaStream_t s) {
+  const int64_t b = std::min<int64_t>((N + kPolyThreads - 1) / kPolyThreads, 152 * 64);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)std::max<int64_t>(1, b));
+  cfg.blockDim = dim3(kPolyThreads);
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl_enabled() ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, poly_kernel<T>, terms, q, N, stage2);
 }
 
-// out = alpha * (in x_mu M) + beta * base for one component, natural layout
+// out_c = alpha * (in_c x_mu M_c) + beta * base_c for every component in one
+// launch (one per component left the GPU with a few dozen CTAs at a time: 20
+// launches of 12.5 us a step on 130 x 72 with three components), natural layout
 // (x_1 fastest): mode 1 is X M^T over the rows of length n_1, mode mu > 1 is
-// M X over the n_mu x (n_1 .. n_{mu-1}) slabs.
+// M X over the n_mu x (n_1 .. n_{mu-1}) slabs.  k: 0 = A, 1 = phi_1, 2 = phi_2.
 template <typename T>
-static cudaError_t mode_one(adr_plan P, int mu, const void* M, const void* MT, const void* in,
-                            void* out, const void* base, double alpha, double beta) {
+static cudaError_t mode_all(adr_plan P, int mu, int k, void* const* in, void* const* out,
+                            void* const* base, double alpha, double beta) {
+  const GeneralState& S = *P->gen;
   const int64_t n = P->n[mu];
   int64_t Q = 1;
-  for (int k = 0; k < mu; ++k) Q *= P->n[k];
+  for (int j = 0; j < mu; ++j) Q *= P->n[j];
   const int64_t Pb = P->N / (n * Q);
   GemmArgs g{};
-  g.ncomp = 1;
+  g.ncomp = S.m;
   g.alpha = alpha;
   g.beta = beta;
-  g.C[0] = out;
-  g.base[0] = base;
-  g.base2[0] = nullptr;
+  for (int c = 0; c < S.m; ++c) {
+    g.C[c] = out[c];
+    g.base[c] = base ? base[c] : nullptr;
+    g.A[c] = mu == 0 ? in[c] : S.op[c][mu][k];
+    g.B[c] = mu == 0 ? S.opT[c][mu][k] : in[c];
+  }
   if (mu == 0) {
-    g.A[0] = in;
-    g.B[0] = MT;
     g.M = (int)Pb;
     g.N = (int)n;
     g.K = (int)n;
     g.lda = g.ldb = g.ldc = n;
     g.batch = 1;
   } else {
-    g.A[0] = M;
-    g.B[0] = in;
     g.M = (int)n;
     g.N = (int)Q;
     g.K = (int)n;
@@ -130,8 +148,8 @@ static cudaError_t mode_one(adr_plan P, int mu, const void* M, const void* MT, c
     g.c_bs = n * Q;
     g.batch = (int)Pb;
   }
-  const double flops = 2.0 * (double)n * (double)P->N;
-  const double bytes = (double)sizeof(T) * (2.0 * P->N + (base ? P->N : 0) + n * n);
+  const double flops = 2.0 * (double)n * (double)P->N * S.m;
+  const double bytes = (double)sizeof(T) * (2.0 * P->N + (base ? P->N : 0) + n * n) * S.m;
   return timed_kernel(P, KC_MODE_SIMT, flops, bytes, [&] { return launch_gemm_simt<T>(g, P->stream); });
 }
 
@@ -143,10 +161,8 @@ static cudaError_t step_general(adr_plan P, void* const* U) {
   const int64_t N = P->N;
   cudaError_t e = cudaSuccess;
   // W_c = sum_mu U_c x_mu A_mu^c
-  for (int c = 0; c < m && e == cudaSuccess; ++c)
-    for (int mu = 0; mu < d && e == cudaSuccess; ++mu)
-      e = mode_one<T>(P, mu, G.op[c][mu][0], G.opT[c][mu][0], U[c], G.w[c], mu ? G.w[c] : nullptr,
-                      1.0, mu ? 1.0 : 0.0);
+  for (int mu = 0; mu < d && e == cudaSuccess; ++mu)
+    e = mode_all<T>(P, mu, 0, U, G.w, mu ? G.w : nullptr, 1.0, mu ? 1.0 : 0.0);
   if (e != cudaSuccess) return e;
   GenPtrs q{};
   for (int c = 0; c < m; ++c) {
@@ -154,35 +170,29 @@ static cudaError_t step_general(adr_plan P, void* const* U) {
     q.u2[c] = G.u2[c];
     q.w[c] = G.w[c];
   }
-  const int gr = grid_of(N);
   e = timed_kernel(P, KC_RHS, (double)N * 8.0 * G.terms.n, (double)sizeof(T) * N * 3 * m, [&] {
-    poly_kernel<T><<<gr, 256, 0, P->stream>>>(G.terms, q, N, 0);
-    return cudaGetLastError();
+    return launch_poly<T>(G.terms, q, N, 0, P->stream);
   });
   if (e != cudaSuccess) return e;
   // U2_c = U_c + tau W_c x_mu phi_1, then the stage-2 pair
-  auto tucker = [&](int c, int k, const void* in, void* out, const void* base, double alpha) {
-    const void* cur = in;
+  auto tucker = [&](int k, void* const* in, void* const* out, void* const* base, double alpha) {
+    void* const* cur = in;
     cudaError_t r = cudaSuccess;
     for (int mu = 0; mu < d && r == cudaSuccess; ++mu) {
       const bool last = mu == d - 1;
-      void* dst = last ? out : ((mu & 1) ? G.t1[c] : G.t0[c]);
-      r = mode_one<T>(P, mu, G.op[c][mu][k], G.opT[c][mu][k], cur, dst, last ? base : nullptr,
-                      last ? alpha : 1.0, last ? 1.0 : 0.0);
+      void* const* dst = last ? out : ((mu & 1) ? G.t1 : G.t0);
+      r = mode_all<T>(P, mu, k, cur, dst, last ? base : nullptr, last ? alpha : 1.0, last ? 1.0 : 0.0);
       cur = dst;
     }
     return r;
   };
-  for (int c = 0; c < m && e == cudaSuccess; ++c) e = tucker(c, 1, G.w[c], G.u2[c], U[c], tau);
+  e = tucker(1, G.w, G.u2, U, tau);
   if (e != cudaSuccess) return e;
   e = timed_kernel(P, KC_RDIFF, (double)N * 16.0 * G.terms.n, (double)sizeof(T) * N * 3 * m, [&] {
-    poly_kernel<T><<<gr, 256, 0, P->stream>>>(G.terms, q, N, 1);
-    return cudaGetLastError();
+    return launch_poly<T>(G.terms, q, N, 1, P->stream);
   });
   if (e != cudaSuccess) return e;
-  const double c2 = ldexp(tau, d - 1);
-  for (int c = 0; c < m && e == cudaSuccess; ++c) e = tucker(c, 2, G.w[c], U[c], G.u2[c], c2);
-  return e;
+  return tucker(2, G.w, U, G.u2, ldexp(tau, d - 1));
 }
 
 cudaError_t general_step(adr_plan P, void* const* U) {

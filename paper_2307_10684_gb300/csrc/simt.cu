@@ -5,15 +5,45 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <math.h>
+
+#include <algorithm>
+
 #include "adr_internal.h"
 #include "pointwise.cuh"
 
 namespace adr {
 
+// Programmatic dependent launch: a kernel of a step waits for its predecessors
+// before it touches memory, and lets the next one be scheduled when its own
+// work is nearly done.  Not at its start: the next kernel's blocks would then
+// be placed while this one's hold most SMs, several to each that is free
+// (FP64 64^2, 128 blocks a launch: 28.5 us a step so, 19.5 with the late
+// trigger, 30 without programmatic launches; 128^2 54.8 / 49.7 / 60.3).
+__device__ __forceinline__ void simt_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void simt_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <typename... KArgs, typename... Args>
+static cudaError_t simt_launch(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                               Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = pdl_enabled() ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, kern, KArgs(args)...);
+}
+
 template <typename T>
 __global__ void __launch_bounds__(128) rhs_kernel(PointwiseArgsT<T> a, const T* __restrict__ u,
                                                   const T* __restrict__ v, T* __restrict__ wu,
                                                   T* __restrict__ wv) {
+  simt_wait();
   const int i1 = blockIdx.x * blockDim.x + threadIdx.x;
   if (i1 >= (int)a.n[0]) return;
   const int i2 = blockIdx.y, i3 = blockIdx.z;
@@ -22,6 +52,7 @@ __global__ void __launch_bounds__(128) rhs_kernel(PointwiseArgsT<T> a, const T* 
   rhs_point<T>(a, u, v, idx, i1, i2, i3, x, y);
   wu[idx] = x;
   wv[idx] = y;
+  simt_trigger();
 }
 
 template <typename T>
@@ -30,10 +61,12 @@ __global__ void __launch_bounds__(256) rdiff_kernel(PointwiseArgsT<T> a, const T
                                                     const T* __restrict__ u2,
                                                     const T* __restrict__ v2, T* __restrict__ du,
                                                     T* __restrict__ dv) {
+  simt_wait();
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < a.N;
        idx += (int64_t)gridDim.x * blockDim.x) {
     react_diff<T>(a.rx, u[idx], v[idx], u2[idx], v2[idx], du[idx], dv[idx]);
   }
+  simt_trigger();
 }
 
 // Lawson2b (Eq. 7) pointwise stages: x = u + scale G^u(u, v) (both
@@ -42,6 +75,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) lawson_pre_kernel(PointwiseArgsT<T> a, const T* __restrict__ u,
                                                          const T* __restrict__ v, T scale,
                                                          T* __restrict__ xu, T* __restrict__ xv) {
+  simt_wait();
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < a.N;
        idx += (int64_t)gridDim.x * blockDim.x) {
     T gu, gv;
@@ -50,6 +84,7 @@ __global__ void __launch_bounds__(256) lawson_pre_kernel(PointwiseArgsT<T> a, co
     xu[idx] = uu + scale * gu;
     xv[idx] = vv + scale * gv;
   }
+  simt_trigger();
 }
 
 template <typename T>
@@ -57,6 +92,7 @@ __global__ void __launch_bounds__(256) lawson_post_kernel(PointwiseArgsT<T> a,
                                                           const T* __restrict__ u2,
                                                           const T* __restrict__ v2, T scale,
                                                           T* __restrict__ u, T* __restrict__ v) {
+  simt_wait();
   for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < a.N;
        idx += (int64_t)gridDim.x * blockDim.x) {
     T gu, gv;
@@ -64,41 +100,43 @@ __global__ void __launch_bounds__(256) lawson_post_kernel(PointwiseArgsT<T> a,
     u[idx] += scale * gu;
     v[idx] += scale * gv;
   }
+  simt_trigger();
 }
 
-static int pointwise_grid(int64_t N) {
-  int64_t b = (N + 255) / 256;
-  const int64_t cap = 152 * 16;
-  return (int)(b < cap ? (b < 1 ? 1 : b) : cap);
+// Threads of a flat block: 64 in FP64, so that a grid of a few thousand points
+// covers all SMs (two FP64 operations a clock each).
+template <typename T>
+constexpr int kFlatThreads = sizeof(T) == 8 ? 64 : 256;
+template <typename T>
+static dim3 pointwise_grid(int64_t N) {
+  const int64_t b = (N + kFlatThreads<T> - 1) / kFlatThreads<T>;
+  const int64_t cap = 152 * 16 * (256 / kFlatThreads<T>);
+  return dim3((unsigned)(b < cap ? (b < 1 ? 1 : b) : cap));
 }
 
 template <typename T>
 cudaError_t launch_rhs(const PointwiseArgsT<T>& a, const T* u, const T* v, T* wu, T* wv,
                        cudaStream_t s) {
   dim3 grid((unsigned)((a.n[0] + 127) / 128), (unsigned)a.n[1], (unsigned)(a.d == 3 ? a.n[2] : 1));
-  rhs_kernel<T><<<grid, 128, 0, s>>>(a, u, v, wu, wv);
-  return cudaGetLastError();
+  return simt_launch(rhs_kernel<T>, grid, dim3(128), 0, s, a, u, v, wu, wv);
 }
 
 template <typename T>
 cudaError_t launch_rdiff(const PointwiseArgsT<T>& a, const T* u, const T* v, const T* u2, const T* v2,
                          T* du, T* dv, cudaStream_t s) {
-  rdiff_kernel<T><<<pointwise_grid(a.N), 256, 0, s>>>(a, u, v, u2, v2, du, dv);
-  return cudaGetLastError();
+  return simt_launch(rdiff_kernel<T>, pointwise_grid<T>(a.N), dim3(kFlatThreads<T>), 0, s, a, u, v, u2, v2, du, dv);
 }
 
 template <typename T>
 cudaError_t launch_lawson_pre(const PointwiseArgsT<T>& a, const T* u, const T* v, T scale, T* xu,
                               T* xv, cudaStream_t s) {
-  lawson_pre_kernel<T><<<pointwise_grid(a.N), 256, 0, s>>>(a, u, v, scale, xu, xv);
-  return cudaGetLastError();
+  return simt_launch(lawson_pre_kernel<T>, pointwise_grid<T>(a.N), dim3(kFlatThreads<T>), 0, s, a, u, v, scale, xu, xv);
 }
 
 template <typename T>
 cudaError_t launch_lawson_post(const PointwiseArgsT<T>& a, const T* u2, const T* v2, T scale, T* u,
                                T* v, cudaStream_t s) {
-  lawson_post_kernel<T><<<pointwise_grid(a.N), 256, 0, s>>>(a, u2, v2, scale, u, v);
-  return cudaGetLastError();
+  return simt_launch(lawson_post_kernel<T>, pointwise_grid<T>(a.N), dim3(kFlatThreads<T>), 0, s, a, u2, v2, scale, u, v);
 }
 
 template cudaError_t launch_lawson_pre<float>(const PointwiseArgsT<float>&, const float*,
@@ -123,118 +161,156 @@ template cudaError_t launch_rdiff<double>(const PointwiseArgsT<double>&, const d
                                           cudaStream_t);
 
 // ---------------------------------------------------------------- GEMM
-// Tile configuration: 256 threads as a 16 x 16 grid; each thread owns a
-// TM x TN block of C split into 4-wide groups spread over the tile so that
-// shared-memory reads are conflict free.
-template <typename T>
-struct SimtTile;
-template <>
-struct SimtTile<float> {
-  static constexpr int BM = 128, BN = 128, BK = 8, TM = 8, TN = 8;
+// One CTA computes a BM x BN tile of C, a thread a TM x TN block of it.  A and
+// B panels of KC values of K go through ST shared-memory stages by cp.async,
+// ST - 1 of them requested ahead: the products of the small plans (K of a few
+// dozen to a few hundred) are one or two stages long, so a launch pays one
+// memory round trip instead of one per 8 values of K.  Every output is one
+// chain of FMAs over k = 0, 1, ..., K - 1, whatever the tile (KS such chains
+// where the tile's K is split).
+__device__ __forceinline__ uint32_t smem_addr(const void* p) {
+  return (uint32_t)__cvta_generic_to_shared(p);
+}
+// bytes <= B are copied, the rest of the B bytes zero-filled
+template <int B>
+__device__ __forceinline__ void cp_async(void* dst, const void* src, int bytes) {
+  if constexpr (B == 16)
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_addr(dst)), "l"(src), "r"(bytes)
+                 : "memory");
+  else
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2, %3;" ::"r"(smem_addr(dst)), "l"(src), "n"(B),
+                 "r"(bytes)
+                 : "memory");
+}
+// rows x cols values of a row-major matrix (leading dimension ld) from src
+// into dst (row pitch PITCH), rows and columns beyond nr, nc as zeros
+template <typename T, int ROWS, int COLS, int PITCH, int THREADS, bool VEC>
+__device__ __forceinline__ void load_panel(T* dst, const T* src, int64_t ld, int nr, int nc) {
+  constexpr int V = VEC ? 16 / (int)sizeof(T) : 1, CV = COLS / V;
+#pragma unroll
+  for (int i0 = 0; i0 < ROWS * CV; i0 += THREADS) {
+    const int i = i0 + threadIdx.x;
+    if (ROWS * CV % THREADS != 0 && i >= ROWS * CV) break;
+    const int r = i / CV, c = i % CV * V;
+    const int n = r < nr ? min(V, max(0, nc - c)) : 0;
+    cp_async<V * (int)sizeof(T)>(dst + r * PITCH + c, n > 0 ? src + r * ld + c : src, n * (int)sizeof(T));
+  }
+}
+
+// KS: groups of threads that share the tile's K (each takes every KS-th run
+// of V values of a stage); their sums are added in order at the end.
+template <typename T, int BM_, int BN_, int TM_, int TN_, int KC_, int ST_, int KS_ = 1>
+struct GemmCfg {
+  static constexpr int BM = BM_, BN = BN_, TM = TM_, TN = TN_, KC = KC_, ST = ST_, KS = KS_;
+  static constexpr int V = 16 / (int)sizeof(T);            // values per 16 bytes
+  static constexpr int GROUP = (BM / TM) * (BN / TN);      // threads of one group
+  static constexpr int THREADS = GROUP * KS;
+  static constexpr int PA = KC + V, PB = BN + V;           // row pitches
+  static constexpr int STAGE = BM * PA + KC * PB;          // values
+  static constexpr int SMEM = ST * STAGE * (int)sizeof(T);
 };
-template <>
-struct SimtTile<double> {
-  static constexpr int BM = 64, BN = 64, BK = 8, TM = 4, TN = 4;
-};
 
-template <typename T>
-__global__ void __launch_bounds__(256) gemm_simt_kernel(GemmArgs g) {
-  using Cfg = SimtTile<T>;
-  constexpr int BM = Cfg::BM, BN = Cfg::BN, BK = Cfg::BK, TM = Cfg::TM, TN = Cfg::TN;
-  constexpr int LA = BM * BK / 256;  // A elements loaded per thread (along k)
-  constexpr int LB = BK * BN / 256;  // B elements loaded per thread (along n)
-  constexpr int RS = TM / 4, CS = TN / 4;
-
-  __shared__ __align__(16) T As[2][BK][BM];
-  __shared__ __align__(16) T Bs[2][BK][BN];
-
+template <typename T, typename C>
+__global__ void __launch_bounds__(C::THREADS) gemm_kernel(const __grid_constant__ GemmArgs g) {
+  constexpr int BM = C::BM, BN = C::BN, TM = C::TM, TN = C::TN, KC = C::KC, ST = C::ST, V = C::V;
+  extern __shared__ __align__(16) uint8_t smem_raw[];
+  T* sm = reinterpret_cast<T*>(smem_raw);
+  simt_wait();
   const int z = blockIdx.z;
   const int comp = z / g.batch;
   const int p = z - comp * g.batch;
-  const T* __restrict__ A = (const T*)g.A[comp] + (int64_t)p * g.a_bs;
-  const T* __restrict__ B = (const T*)g.B[comp] + (int64_t)p * g.b_bs;
   const int m0 = blockIdx.y * BM, n0 = blockIdx.x * BN;
-  const int t = threadIdx.x;
-  const int tx = t & 15, ty = t >> 4;
-
-  // load coordinates
-  const int a_row = t / (BK / LA), a_k = (t % (BK / LA)) * LA;
-  const int b_k = t / (BN / LB), b_n = (t % (BN / LB)) * LB;
-
-  T ra[LA], rb[LB];
-  auto load_tiles = [&](int k0) {
-    const int gr = m0 + a_row;
-#pragma unroll
-    for (int i = 0; i < LA; ++i) {
-      const int gk = k0 + a_k + i;
-      ra[i] = (gr < g.M && gk < g.K) ? A[(int64_t)gr * g.lda + gk] : (T)0;
+  const T* __restrict__ A = (const T*)g.A[comp] + (int64_t)p * g.a_bs + (int64_t)m0 * g.lda;
+  const T* __restrict__ B = (const T*)g.B[comp] + (int64_t)p * g.b_bs + n0;
+  // 16-byte copies where every row of the operand starts on 16 bytes
+  const bool va = (((uintptr_t)A | (uintptr_t)(g.lda * (int64_t)sizeof(T))) & 15) == 0;
+  const bool vb = (((uintptr_t)B | (uintptr_t)(g.ldb * (int64_t)sizeof(T))) & 15) == 0;
+  const int nk = (g.K + KC - 1) / KC;
+  auto load = [&](int kt) {
+    if (kt < nk) {
+      T* st = sm + kt % ST * C::STAGE;
+      const int k0 = kt * KC;
+      if (va)
+        load_panel<T, BM, KC, C::PA, C::THREADS, true>(st, A + k0, g.lda, g.M - m0, g.K - k0);
+      else
+        load_panel<T, BM, KC, C::PA, C::THREADS, false>(st, A + k0, g.lda, g.M - m0, g.K - k0);
+      T* sb = st + BM * C::PA;
+      if (vb)
+        load_panel<T, KC, BN, C::PB, C::THREADS, true>(sb, B + (int64_t)k0 * g.ldb, g.ldb, g.K - k0, g.N - n0);
+      else
+        load_panel<T, KC, BN, C::PB, C::THREADS, false>(sb, B + (int64_t)k0 * g.ldb, g.ldb, g.K - k0, g.N - n0);
     }
-    const int gk = k0 + b_k;
-#pragma unroll
-    for (int i = 0; i < LB; ++i) {
-      const int gn = n0 + b_n + i;
-      rb[i] = (gk < g.K && gn < g.N) ? B[(int64_t)gk * g.ldb + gn] : (T)0;
-    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
   };
-  auto store_tiles = [&](int buf) {
-#pragma unroll
-    for (int i = 0; i < LA; ++i) As[buf][a_k + i][a_row] = ra[i];
-#pragma unroll
-    for (int i = 0; i < LB; ++i) Bs[buf][b_k][b_n + i] = rb[i];
-  };
-
+  const int kg = threadIdx.x / C::GROUP, gt = threadIdx.x % C::GROUP;
+  const int tx = gt % (BN / TN), ty = gt / (BN / TN);
+  // a thread's columns: groups of min(TN, 4) neighbours spread over the tile;
+  // its rows: BM / TM apart
+  constexpr int G = TN < 4 ? TN : 4;
+  auto col = [&](int j) { return (j / G) * (BN / (TN / G)) + tx * G + j % G; };
+  auto row = [&](int i) { return i * (BM / TM) + ty; };
   T acc[TM][TN];
 #pragma unroll
   for (int i = 0; i < TM; ++i)
 #pragma unroll
     for (int j = 0; j < TN; ++j) acc[i][j] = (T)0;
-
-  load_tiles(0);
-  store_tiles(0);
-  __syncthreads();
-
-  const int ktiles = (g.K + BK - 1) / BK;
-  for (int kt = 0; kt < ktiles; ++kt) {
-    const int cur = kt & 1;
-    if (kt + 1 < ktiles) load_tiles((kt + 1) * BK);
 #pragma unroll
-    for (int kk = 0; kk < BK; ++kk) {
-      T a[TM], b[TN];
-#pragma unroll
-      for (int r = 0; r < RS; ++r)
-#pragma unroll
-        for (int i = 0; i < 4; ++i) a[r * 4 + i] = As[cur][kk][r * (BM / RS) + ty * 4 + i];
-#pragma unroll
-      for (int c = 0; c < CS; ++c)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) b[c * 4 + j] = Bs[cur][kk][c * (BN / CS) + tx * 4 + j];
+  for (int s = 0; s < ST - 1; ++s) load(s);
+  for (int kt = 0; kt < nk; ++kt) {
+    asm volatile("cp.async.wait_group %0;" ::"n"(ST - 2) : "memory");
+    __syncthreads();  // stage kt landed; stage kt - 1 is read by nobody any more
+    load(kt + ST - 1);
+    const T* as = sm + kt % ST * C::STAGE;
+    const T* bs = as + BM * C::PA;
+    const int kend = min(KC, g.K - kt * KC);
+#pragma unroll 2
+    for (int k = kg * V; k < kend; k += C::KS * V) {
+      T a[TM][V], b[V][TN];
 #pragma unroll
       for (int i = 0; i < TM; ++i)
+        *reinterpret_cast<float4*>(&a[i][0]) = *reinterpret_cast<const float4*>(as + row(i) * C::PA + k);
 #pragma unroll
-        for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i], b[j], acc[i][j]);
+      for (int q = 0; q < V; ++q)
+#pragma unroll
+        for (int j = 0; j < TN; j += G) {
+          const T* src = bs + (k + q) * C::PB + col(j);
+          if constexpr (G * sizeof(T) == 16)
+            *reinterpret_cast<float4*>(&b[q][j]) = *reinterpret_cast<const float4*>(src);
+          else
+#pragma unroll
+            for (int e = 0; e < G; ++e) b[q][j + e] = src[e];
+        }
+#pragma unroll
+      for (int q = 0; q < V; ++q)
+#pragma unroll
+        for (int i = 0; i < TM; ++i)
+#pragma unroll
+          for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i][q], b[q][j], acc[i][j]);
     }
-    if (kt + 1 < ktiles) {
-      store_tiles(cur ^ 1);
-    }
-    __syncthreads();
   }
-
-  // epilogue
-  T* __restrict__ C = (T*)g.C[comp] + (int64_t)p * g.c_bs;
-  const T* __restrict__ base = g.base[comp] ? (const T*)g.base[comp] + (int64_t)p * g.c_bs : nullptr;
-  const T* __restrict__ base2 =
-      g.base2[comp] ? (const T*)g.base2[comp] + (int64_t)p * g.c_bs : nullptr;
+  simt_trigger();
+  if constexpr (C::KS > 1) {
+    static_assert(TM == 1 && TN == 1, "split contractions: one output a thread");
+    __syncthreads();
+    sm[threadIdx.x] = acc[0][0];
+    __syncthreads();
+    if (kg != 0) return;
+#pragma unroll
+    for (int q = 1; q < C::KS; ++q) acc[0][0] += sm[q * C::GROUP + gt];
+  }
+  // out = alpha acc + beta base + beta2 base2
+  T* __restrict__ Co = (T*)g.C[comp] + (int64_t)p * g.c_bs;
+  const T* base = g.base[comp] ? (const T*)g.base[comp] + (int64_t)p * g.c_bs : nullptr;
+  const T* base2 = g.base2[comp] ? (const T*)g.base2[comp] + (int64_t)p * g.c_bs : nullptr;
   const T alpha = (T)g.alpha, beta = (T)g.beta, beta2 = (T)g.beta2;
 #pragma unroll
   for (int i = 0; i < TM; ++i) {
-    const int r = m0 + (i / 4) * (BM / RS) + ty * 4 + (i % 4);
+    const int r = m0 + row(i);
     if (r >= g.M) continue;
-    // gather the row's epilogue inputs before any store (C may share no
-    // memory with base/base2, but the compiler cannot assume it)
-    T extra[TN];
+    T extra[TN];  // the row's base values before any store (C may be the base)
 #pragma unroll
     for (int j = 0; j < TN; ++j) {
-      const int c = n0 + (j / 4) * (BN / CS) + tx * 4 + (j % 4);
+      const int c = n0 + col(j);
       const int64_t o = (int64_t)r * g.ldc + c;
       T x = (T)0;
       if (c < g.N) {
@@ -245,68 +321,86 @@ __global__ void __launch_bounds__(256) gemm_simt_kernel(GemmArgs g) {
     }
 #pragma unroll
     for (int j = 0; j < TN; ++j) {
-      const int c = n0 + (j / 4) * (BN / CS) + tx * 4 + (j % 4);
-      if (c < g.N) C[(int64_t)r * g.ldc + c] = alpha * acc[i][j] + extra[j];
+      const int c = n0 + col(j);
+      if (c < g.N) Co[(int64_t)r * g.ldc + c] = alpha * acc[i][j] + extra[j];
     }
   }
 }
 
-// Small-problem variant: an 8 x 8 output tile per 64-thread CTA, one output
-// per thread.  Used when the register-blocked kernel would leave most SMs
-// idle (GB300 runs FP64 at about two FMAs per clock per SM, so a 64^3
-// product on a single SM takes tens of microseconds).
-template <typename T>
-__global__ void __launch_bounds__(64) gemm_small_kernel(GemmArgs g) {
-  constexpr int TS = 8;
-  __shared__ T As[TS][TS + 1];
-  __shared__ T Bs[TS][TS + 1];
-  const int z = blockIdx.z;
-  const int comp = z / g.batch;
-  const int p = z - comp * g.batch;
-  const T* __restrict__ A = (const T*)g.A[comp] + (int64_t)p * g.a_bs;
-  const T* __restrict__ B = (const T*)g.B[comp] + (int64_t)p * g.b_bs;
-  const int tx = threadIdx.x & 7, ty = threadIdx.x >> 3;
-  const int r = blockIdx.y * TS + ty, c = blockIdx.x * TS + tx;
-  T acc = (T)0;
-  for (int k0 = 0; k0 < g.K; k0 += TS) {
-    As[ty][tx] = (r < g.M && k0 + tx < g.K) ? A[(int64_t)r * g.lda + k0 + tx] : (T)0;
-    Bs[ty][tx] = (k0 + ty < g.K && c < g.N) ? B[(int64_t)(k0 + ty) * g.ldb + c] : (T)0;
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < TS; ++k) acc = fma(As[ty][k], Bs[k][tx], acc);
-    __syncthreads();
-  }
-  if (r < g.M && c < g.N) {
-    const int64_t o = (int64_t)r * g.ldc + c;
-    T* __restrict__ C = (T*)g.C[comp] + (int64_t)p * g.c_bs;
-    T x = (T)g.alpha * acc;
-    if (g.base[comp]) x += (T)g.beta * ((const T*)g.base[comp] + (int64_t)p * g.c_bs)[o];
-    if (g.base2[comp]) x += (T)g.beta2 * ((const T*)g.base2[comp] + (int64_t)p * g.c_bs)[o];
-    C[o] = x;
-  }
-}
-
-template <typename T>
-cudaError_t launch_gemm_simt(const GemmArgs& g, cudaStream_t s) {
-  using Cfg = SimtTile<T>;
-  if (g.M <= 0 || g.N <= 0) return cudaSuccess;
-  dim3 grid((g.N + Cfg::BN - 1) / Cfg::BN, (g.M + Cfg::BM - 1) / Cfg::BM, g.batch * g.ncomp);
-  // FP64 runs ~40x slower per SM than FP32, so FP64 products spread over
-  // small tiles whenever the large tiles leave SMs idle; FP32 only for tiny
-  // problems
-  const int64_t min_ctas = sizeof(T) == 8 ? 152 : 32;
-  if ((int64_t)grid.x * grid.y * grid.z < min_ctas) {
-    dim3 sg((g.N + 7) / 8, (g.M + 7) / 8, g.batch * g.ncomp);
-    if (sg.y > 65535 || sg.z > 65535) return cudaErrorInvalidConfiguration;
-    gemm_small_kernel<T><<<sg, 64, 0, s>>>(g);
-    return cudaGetLastError();
-  }
+template <typename T, typename C>
+static cudaError_t run_gemm(const GemmArgs& g, cudaStream_t s) {
+  const dim3 grid((g.N + C::BN - 1) / C::BN, (g.M + C::BM - 1) / C::BM, g.batch * g.ncomp);
   if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidConfiguration;
-  gemm_simt_kernel<T><<<grid, 256, 0, s>>>(g);
-  return cudaGetLastError();
+  // no more tiles than SMs: over half an SM's shared memory, so that no two
+  // blocks share an SM (FP64 64^2 18.0 us a step, 19.5 without)
+  constexpr int kAlone = C::SMEM > 115 * 1024 ? C::SMEM : 115 * 1024;
+  const int smem = (int64_t)grid.x * grid.y * grid.z <= 152 ? kAlone : C::SMEM;
+  if (smem > 48 * 1024) {  // an attribute of the current device's kernel, the same from every thread
+    const cudaError_t e =
+        cudaFuncSetAttribute(gemm_kernel<T, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAlone);
+    if (e != cudaSuccess) return e;
+  }
+  return simt_launch(gemm_kernel<T, C>, grid, dim3(C::THREADS), smem, s, g);
 }
 
-template cudaError_t launch_gemm_simt<float>(const GemmArgs&, cudaStream_t);
-template cudaError_t launch_gemm_simt<double>(const GemmArgs&, cudaStream_t);
+// FP64: an SM retires two FMAs a clock (a warp's takes one of its four units
+// 64 clocks), so what counts is that the tiles divide evenly over the SMs and
+// that every unit has a warp: 8 x 8 tiles, K split two ways; four ways where
+// an SM has one tile at most.  us a step, ETD2RKds, 64 x 64 tiles with an 8 x 8
+// kernel for small plans (before) / K in two / in four:
+//   32^2 33.8 / 15.6 / 15.2   64^2 44.0 / 19.0 / 17.8   128^2 74.7 / 47.9 / 49.4
+//   256^2 276 / 252 / 251     512^2 1821 / 1781 / 1795  1024^2 16567 / 13920 / 13986
+//   32^3 60.5 / 46.0 / 51.2   64^3 415 / 403 / 414      160^3 17024 / 13469 / 13677
+// (16 x 16 tiles: 48.8, 280, 1835, 13917; 45.3, 403, 13330.)  What is left
+// above the FMA time (256^2: 232 us) is the pointwise kernels and launches.
+template <>
+cudaError_t launch_gemm_simt<double>(const GemmArgs& g, cudaStream_t s) {
+  if (g.M <= 0 || g.N <= 0) return cudaSuccess;
+  using S8 = GemmCfg<double, 8, 8, 1, 1, 64, 3, 2>;
+  using S8x4 = GemmCfg<double, 8, 8, 1, 1, 64, 3, 4>;
+  using S64 = GemmCfg<double, 64, 64, 4, 4, 16, 3>;
+  const int64_t rows = (g.M + 7) / 8;
+  if (rows > 65535) return run_gemm<double, S64>(g, s);  // a launch's limit
+  if (rows * ((g.N + 7) / 8) * g.batch * g.ncomp <= 152) return run_gemm<double, S8x4>(g, s);
+  return run_gemm<double, S8>(g, s);
+}
+
+// FP32: larger blocks per thread reuse more of each shared-memory load, but
+// leave SMs idle sooner.  Clocks of a launch on tiles of configuration C: with
+// w tiles on the fullest SM, `rate` FMAs a clock at w >> h, less where few
+// warps hide each other's latency.
+template <typename C>
+static double gemm_clocks(const GemmArgs& g, double rate, double h) {
+  const double tiles = (double)((g.N + C::BN - 1) / C::BN) * ((g.M + C::BM - 1) / C::BM) * g.batch * g.ncomp;
+  return (ceil(tiles / 152.0) + h) * C::BM * C::BN * g.K / rate;
+}
+
+// Rates and h from us a step, 128 x 128 tiles (before) / 32 x 32 / 64 x 32 /
+// 64 x 64 / 128 x 128:
+//   128^2 42.0 / 20.7 / 27.6 / 34.8 / 90.5    384^2 231 / 57.6 / 55.7 / 75.5 / 213
+//   512^2 361 / 131 / 109 / 97.2 / 275        1024^2 716 / 814 / 569 / 551 / 527
+//   1500^2 2203 / 2527 / 1542 / 1571 / 1365   64^3 107 / 54.4 / 47.1 / 42.9 / 79.6
+//   96^3 191 / 159 / 128 / 134 / 139          160^3 1271 / 916 / 664 / 685 / 916
+template <>
+cudaError_t launch_gemm_simt<float>(const GemmArgs& g, cudaStream_t s) {
+  if (g.M <= 0 || g.N <= 0) return cudaSuccess;
+  using S32 = GemmCfg<float, 32, 32, 2, 2, 64, 3>;
+  using S64n = GemmCfg<float, 64, 32, 4, 4, 32, 3>;
+  using S64 = GemmCfg<float, 64, 64, 4, 4, 32, 3>;
+  using S128 = GemmCfg<float, 128, 128, 8, 8, 16, 3>;
+  const double c[4] = {gemm_clocks<S32>(g, 40.0, 0.5), gemm_clocks<S64n>(g, 62.0, 0.65),
+                       gemm_clocks<S64>(g, 72.0, 0.4), gemm_clocks<S128>(g, 82.0, 0.1)};
+  int best = 3;
+  for (int i = 2; i >= 0; --i) {
+    const int64_t bm = i == 0 ? 32 : 64;
+    if (c[i] < c[best] && (g.M + bm - 1) / bm <= 65535) best = i;
+  }
+  switch (best) {
+    case 0: return run_gemm<float, S32>(g, s);
+    case 1: return run_gemm<float, S64n>(g, s);
+    case 2: return run_gemm<float, S64>(g, s);
+    default: return run_gemm<float, S128>(g, s);
+  }
+}
 
 }  // namespace adr
