@@ -387,7 +387,7 @@ extern "C" adr_status adr_plan_create_tuned(const adr_problem* problem, const ad
   const size_t sb = (size_t)P->N * P->esize;
   PLAN_TRY(plan_alloc(P, &P->u2, sb));
   PLAN_TRY(plan_alloc(P, &P->v2, sb));
-  for (int c = 0; c < 2; ++c) {
+  for (int c = 0; c < 2 && P->prec <= ADR_FP32; ++c) {  // tensor-core plans keep piece buffers instead
     PLAN_TRY(plan_alloc(P, &P->bufA[c], sb));
     PLAN_TRY(plan_alloc(P, &P->bufB[c], sb));
   }

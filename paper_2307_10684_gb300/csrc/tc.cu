@@ -3674,21 +3674,6 @@ cudaError_t tc_prepare(TcOperands* t, int prec, int scheme, int d, const int64_t
                           kVariants[S->variant].cta2 ? bn / 2 : bn, sw, S->fmt);
         if (e != cudaSuccess) return e;
       }
-  // host copies of the supports, ordered on the plan's stream (a copy on the
-  // legacy stream would wait for every other stream's queued work)
-  for (int c = 0; c < 2; ++c)
-    for (int m = 0; m < d; ++m)
-      for (int l = 0; l < 3; ++l)
-        if (!S->hband[c][m][l].empty()) {
-          e = cudaMemcpyAsync(S->hband[c][m][l].data(), S->kband[c][m][l],
-                              sizeof(int2) * S->hband[c][m][l].size(), cudaMemcpyDeviceToHost, s);
-          if (e != cudaSuccess) return e;
-        }
-  e = cudaStreamSynchronize(s);  // the split matrices and the supports' copies are complete
-  if (e != cudaSuccess) return e;
-  // no kernel requested: the library's own choice
-  S->tp = S->fused12 && variant_req < 0 && getenv("ADR_TC_VARIANT") == nullptr && tp_better(S);
-  if (S->tp) S->variant = 0;  // one step sequence for every grid: all group in a batch
   S->lo[0] = S->lo[1] = nullptr;
   S->comp_u = S->comp_v = nullptr;
   S->ind = nullptr;
@@ -3709,6 +3694,22 @@ cudaError_t tc_prepare(TcOperands* t, int prec, int scheme, int d, const int64_t
         if (e != cudaSuccess) return e;
       }
     }
+  // host copies of the supports, ordered on the plan's stream (a copy on the
+  // legacy stream would wait for every other stream's queued work), after the
+  // allocations, which overlap the matrix functions queued on it
+  for (int c = 0; c < 2; ++c)
+    for (int m = 0; m < d; ++m)
+      for (int l = 0; l < 3; ++l)
+        if (!S->hband[c][m][l].empty()) {
+          e = cudaMemcpyAsync(S->hband[c][m][l].data(), S->kband[c][m][l],
+                              sizeof(int2) * S->hband[c][m][l].size(), cudaMemcpyDeviceToHost, s);
+          if (e != cudaSuccess) return e;
+        }
+  e = cudaStreamSynchronize(s);  // the split matrices and the supports' copies are complete
+  if (e != cudaSuccess) return e;
+  // no kernel requested: the library's own choice
+  S->tp = S->fused12 && variant_req < 0 && getenv("ADR_TC_VARIANT") == nullptr && tp_better(S);
+  if (S->tp) S->variant = 0;  // one step sequence for every grid: all group in a batch
   if (S->tp) {
     for (int c = 0; c < 2 && d == 3; ++c)
       if ((e = alloc((void**)&S->mid[c], (size_t)kPieces * 2 * S->N)) != cudaSuccess) return e;
