@@ -3494,10 +3494,13 @@ void tc_free(TcOperands* t) {
 // Whether the first two directions run as the two-pass launch (tp_kernel)
 // rather than with the intermediate in TMEM (tc_fused_kernel).  us a step,
 // tc_fused_kernel / tp_kernel, plain ETD2RKds:
-//   2D  n2 <= 256, up to 32768 points (64^2 19.2 / 23.6, 128^2 25.8 / 30.4):
-//       TMEM, one launch's latency; beyond that (Brusselator 200^2 49.5 / 40.8,
-//       256^2 52.5 / 39.2) two passes: a unit of tc_fused_kernel holds all of
-//       x2, and a row of tiles is one SM's work;
+//   2D  n2 <= 128, up to 32768 points (64^2 19.2 / 23.6, 128^2 25.8 / 30.4,
+//       160 x 128 27.5 / 31.2, 256 x 128 31.2 / 34.3): TMEM, one tile of x2;
+//   2D  n2 <= 256 beyond that and, with two tiles of x2, from 18000 points
+//       (Brusselator 136^2 43.3 / 34.3, 160^2 38.7 / 32.6, 200^2 49.5 / 40.6,
+//       256^2 52.5 / 39.2): two passes: a unit of tc_fused_kernel holds all of
+//       x2, and a row of tiles is one SM's work (smaller grids stay in TMEM
+//       also with two tiles, so that mixed batches of them are one launch);
 //   2D  n2 > 256 and some x2 tile's support wider than the 256 intermediate
 //       columns (384^2 65.7 / 47.1, 512^2 77.0 / 53.1, 1024^2 168 / 83,
 //       FHN 2048 x 1536 160 / 132): the intermediate is computed again for
@@ -3512,7 +3515,7 @@ static bool tp_better(const TcState* S) {
     auto up = [](int64_t n) { return (double)((n + kBM - 1) / kBM * kBM); };
     return S->N <= 10000000 || up(n1) * up(n2) > 1.1 * (double)(n1 * n2);
   }
-  if (n2 <= kFRowsW) return n1 * n2 > 32768;
+  if (n2 <= kFRowsW) return n1 * n2 > (n2 > kBM ? 18000 : 32768);
   if (!S->ksupport) return true;
   for (int c = 0; c < 2; ++c)
     for (int l = 0; l < 3; ++l)

@@ -68,7 +68,8 @@ def run(adr, p, u0, v0, kernel=-1):
 
 @pytest.mark.parametrize("n,model", [
     ((128, 128), wl.FHN), ((136, 8), wl.BRUSSELATOR), ((8, 392), wl.FHN), ((256, 264), wl.SCHNAKENBERG),
-    ((648, 40), wl.FHN), ((40, 16, 200), wl.FHN), ((8, 8, 8), wl.SCHNAKENBERG),
+    ((648, 40), wl.FHN), ((176, 136), wl.BRUSSELATOR), ((264, 200), wl.FHN),
+    ((1032, 64), wl.SCHNAKENBERG), ((40, 16, 200), wl.FHN), ((8, 8, 8), wl.SCHNAKENBERG),
     ((160, 24, 40), wl.BRUSSELATOR), ((72, 264, 16), wl.FHN), ((192, 8, 16), wl.FHN),
     ((200, 16, 24), wl.SCHNAKENBERG), ((264, 8, 16), wl.BRUSSELATOR)])
 @pytest.mark.parametrize("state", [wl.STATE_PLAIN, wl.STATE_COMPENSATED])
