@@ -431,37 +431,56 @@ __device__ __forceinline__ void comp_update(float b, float lo_in, float inc, flo
 
 __device__ __forceinline__ double trap_w(int i, int n) { return (i == 0 || i == n - 1) ? 0.5 : 1.0; }
 
-// Indicator sums (Sec. 4) of one lane's values: sum of w x and of (x - x_prev)^2,
-// kept as FP32 pairs by TwoSum (about 48 bits) and not in FP64: the FP64 pipe
-// retires two operations a clock and SM, and five per value took 40 us of the
-// last product of a 200^2 grid (58 of 118 us a step; 46 with the pairs).
+// Indicator sums (Sec. 4) of one lane's values: sum of w x and of (x - x_prev)^2.
+// Each is kept exactly to some 70 bits as three FP32 words (TwoSum cascades)
+// and not in FP64: the FP64 pipe retires two operations a clock and SM, and
+// five per value took 58 us a step of a 200^2 grid in the two-pass launch
+// (64 monitored steps: 3350 us with FP32 words).
+// Values whose words could overflow or lose bits to the smallest FP32 number
+// (and infinities and NaN) go to FP64 sums beside them.
 struct IndSums {
-  float sh = 0.f, sl = 0.f, dh = 0.f, dl = 0.f;
-  static __device__ __forceinline__ void acc(float& h, float& l, float x) {
-    float s, e;
-    two_sum(h, x, s, e);
-    h = s;
-    l = __fadd_rn(l, e);
+  float s[3] = {0.f, 0.f, 0.f}, q[3] = {0.f, 0.f, 0.f};
+  double sd = 0.0, qd = 0.0;
+  static __device__ __forceinline__ void low(float (&a)[3], float x) {
+    float e;
+    two_sum(a[1], x, a[1], e);
+    a[2] = __fadd_rn(a[2], e);
+  }
+  static __device__ __forceinline__ void acc(float (&a)[3], float x) {
+    float e;
+    two_sum(a[0], x, a[0], e);
+    low(a, e);
   }
   __device__ __forceinline__ void add(float x, float prev, bool edge) {
-    acc(sh, sl, edge ? 0.5f * x : x);
-    float d, de;  // x - prev, exactly d + de
+    float d, de;  // x - prev, exactly d + de; its square d d + 2 d de + de de
     two_sum(x, -prev, d, de);
-    const float p = __fmul_rn(d, d);
-    acc(dh, dl, p);
-    dl = __fadd_rn(dl, __fmaf_rn(__fmul_rn(2.f, d), de, __fmaf_rn(d, d, -p)));
+    // 2^-35: every product below then ends above 2^-149
+    const float ad = fabsf(d);
+    if (fabsf(x) < 0x1p90f && ad < 0x1p40f && (ad >= 0x1p-35f || ad == 0.f)) {
+      acc(s, edge ? 0.5f * x : x);
+      const float p = __fmul_rn(d, d), r = __fmul_rn(2.f * d, de);
+      acc(q, p);
+      low(q, __fmaf_rn(d, d, -p));
+      low(q, r);
+      q[2] = __fadd_rn(q[2], __fmaf_rn(de, de, __fmaf_rn(2.f * d, de, -r)));
+    } else {
+      sd += edge ? 0.5 * (double)x : (double)x;
+      const double dd = (double)x - (double)prev;
+      qd = fma(dd, dd, qd);
+    }
   }
   // adds the warp's sums (lane weight wm) to the step's slot
   __device__ __forceinline__ void flush(double wm, double* ind) const {
-    double sw = wm * ((double)sh + (double)sl), sd = (double)dh + (double)dl;
+    double sw = wm * (sd + ((double)s[0] + ((double)s[1] + (double)s[2])));
+    double sq = qd + ((double)q[0] + ((double)q[1] + (double)q[2]));
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) {
       sw += __shfl_xor_sync(0xffffffffu, sw, off);
-      sd += __shfl_xor_sync(0xffffffffu, sd, off);
+      sq += __shfl_xor_sync(0xffffffffu, sq, off);
     }
     if ((threadIdx.x & 31) == 0) {
       atomicAdd(ind, sw);
-      atomicAdd(ind + 2, sd);
+      atomicAdd(ind + 2, sq);
     }
   }
 };
