@@ -177,13 +177,16 @@ adr_status adr_plan_create(const adr_problem* problem, void* stream, adr_plan* o
 /* Kernel choice of a tensor-core plan (ADR_BF16X3 / ADR_TF32X3), as chosen
  * by adr_autotune.  The paper has no counterpart: it concerns only how the
  * mode products of Eq. 11 are tiled on the GPU, not what they compute.
- *   kernel : -1 = the library's choice from the grid size;
+ *   kernel : -1 = the library's choice from the grid size and the column
+ *            supports (on some grids a launch of two dependent passes that
+ *            no other value takes);
  *            0 = one CTA per 128 x 128 tile, 64-byte swizzle, 4 stages;
  *            1 = one CTA per 128 x 128 tile, 128-byte swizzle, 2 stages;
  *            2 = one CTA per 128 x 64 tile, 64-byte swizzle;
  *            3 / 4 = two-SM (cta_group::2) 256 x 128 tiles, 64- / 128-byte
  *            swizzle.  TF32X3 plans always use 1.
- * Every kernel computes the same products in the same order per output. */
+ * Kernels 0 to 4 compute the same products in the same order per output; the
+ * library's choice may contract over the union of two row groups' supports. */
 typedef struct {
   int32_t kernel;
   int32_t reserved[7];
@@ -218,7 +221,7 @@ adr_status adr_selftest_bounded_wait(void* stream, int32_t arrive, int64_t limit
 /* Autotuner: for a tensor-core problem, builds a plan with each candidate
  * kernel, advances scratch state (allocated here, zero-filled) by 2 + nsteps
  * steps on `stream` and times the last nsteps with CUDA events.  best
- * receives the fastest kernel; ms_per_step[k] the time per step of kernel k
+ * receives the fastest of the kernels 0 to 4; ms_per_step[k] the time per step of kernel k
  * (-1 when k is not a candidate or failed).  For FP32 / FP64 problems there
  * is nothing to tune: best->kernel = -1 and every entry is -1.  Synchronous;
  * allocates and frees device memory.  nsteps in [1, 1024]. */
