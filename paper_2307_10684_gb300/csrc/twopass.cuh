@@ -142,8 +142,9 @@ __device__ __forceinline__ int tp_slab_tiles(int s, int r) {
   return ((s + 1) * r - 1) / kBM - s * r / kBM + 1;
 }
 // Waits (bounded) until the x1 tiles that an x2 tile reads are complete.
-// seen: the last (component, slab, column tile) found complete by this thread.
-__device__ __forceinline__ bool tp_wait_dep(const TpUnit& w, int& seen) {
+// seen: the last counter found complete by this thread (its address: in a batch
+// every solve has counters of its own, so an index would not tell two apart).
+__device__ __forceinline__ bool tp_wait_dep(const TpUnit& w, const uint32_t*& seen) {
   const TpPass* d = w.d;
   const int m0 = w.mt * kBM, m1 = min(m0 + kBM, d->M) - 1;
   int s0 = 0, s1 = 0, t0 = 0, t1 = 0;
@@ -159,10 +160,10 @@ __device__ __forceinline__ bool tp_wait_dep(const TpUnit& w, int& seen) {
   bool fresh = false;
   for (int s = s0; s <= s1; ++s) {
     const uint32_t want = (uint32_t)(d->dep_want * tp_slab_tiles(s, d->dep_r));
-    const int row = (w.c * d->slabs + s) * d->dep_tn;
+    const uint32_t* row = d->dep + (w.c * d->slabs + s) * d->dep_tn;
     for (int t = t0; t <= t1; ++t) {
       if (row + t == seen) continue;
-      while (ld_acquire(d->dep + row + t) < want)
+      while (ld_acquire(row + t) < want)
         if (globaltimer() - start > kWaitNs) return false;
       seen = row + t;
       fresh = true;
@@ -286,7 +287,7 @@ __global__ void __launch_bounds__(EPI == 0 ? 1024 : kTpThreads, 1) tp_kernel(con
     // is let in and only this launch adds to them, so neither the claims nor
     // the waits for x1 tiles wait for the previous kernel
     if (dynamic && L.clear) pdl_wait();
-    int seen = -1;
+    const uint32_t* seen = nullptr;
     uint32_t t = blockIdx.x;
     for (uint32_t k = 0;; ++k, t += gridDim.x) {
       TpUnit w;
