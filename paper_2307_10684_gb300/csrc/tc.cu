@@ -2043,8 +2043,8 @@ struct PwLaunch {
   const int* bstart;   // [nsolves + 1] prefix sums of this kernel's blocks (desc non-null)
   int nsolves;
   int* err;            // device error word (bounded waits)
-  uint32_t* ctl;       // claims and counters of the two-pass launch that follows (or null),
-  int nctl;            // cleared here
+  uint32_t* ctl;       // a two-pass launch follows: the other control set (or null), cleared here
+  int nctl;
 };
 
 constexpr int kPwThreads = 256;
@@ -2060,17 +2060,17 @@ constexpr int kFlatPerBlock = kPwThreads * 4 * kFlatVec;
 // home = the descriptor where it lives (launch parameter or device memory),
 // from where tensor maps must be read.
 // The next kernel is let in at once; if it is a two-pass launch, only when
-// the previous operator is complete and its claims and counters are cleared,
-// because it claims units before this kernel has finished.
+// the previous operator is complete, because it claims units before this
+// kernel has finished.  Its own control set (claims and counters) was cleared
+// by the row kernel before the previous operator: launch_dependents orders no
+// memory, so nothing that this kernel writes may be read before the wait of
+// the next.  This one clears the set that the previous operator has used.
 __device__ __forceinline__ void pw_open(const PwLaunch& L) {
   pdl_wait();
   if (L.ctl == nullptr) return;
-  if (blockIdx.x == 0) {
-    for (int i = threadIdx.x; i < L.nctl; i += blockDim.x) L.ctl[i] = 0u;
-    __threadfence();
-    __syncthreads();
-  }
   pdl_trigger();
+  if (blockIdx.x == 0)
+    for (int i = threadIdx.x; i < L.nctl; i += blockDim.x) L.ctl[i] = 0u;
 }
 __device__ __forceinline__ const PwDesc* block_desc(const PwLaunch& L, PwDesc* sd, int& lb,
                                                     const PwDesc** home = nullptr) {
@@ -3109,7 +3109,8 @@ struct TcState {
   // two-pass launches (twopass.cuh)
   int tp;
   __nv_bfloat16* mid[2];                  // 3D: output pieces of the two-pass launch
-  uint32_t* tpctl;                        // its claims and dependency counters
+  uint32_t* tpctl;                        // two control sets: claims and dependency counters
+  int tpset;                              // words of a set
   std::vector<TpOp> h_op;                 // [passes]
 };
 
@@ -3371,11 +3372,13 @@ static TpGeo tp_geo(const TcState* S, int mu, int ell, double share) {
   return g;
 }
 static int tp_slabs(const TcState* S) { return S->d == 3 ? (int)S->n[2] : 1; }
-// Dependency counters of the two-pass launch at the narrowest tiles.
-static int64_t tp_dep_words_max(const TcState* S) {
-  return 2 * (int64_t)tp_slabs(S) * ((S->n[0] + 31) / 32 + 8);
-}
 static int tp_npass(const TcPass& ps) { return ps.fused ? 2 : 1; }
+// Control set of pass p: a step's two operators take turns.
+static int tp_set(const TcState* S, int p) {
+  int k = 0;
+  for (int i = 0; i < p; ++i) k += S->passes[i].fused;
+  return k & 1;
+}
 
 // The descriptors of one launch (dep: this solve's counters).
 static cudaError_t make_tp(const TcState* S, const adr_plan_s* P, const TcPass& ps, float* u, float* v,
@@ -3735,9 +3738,9 @@ cudaError_t tc_prepare(TcOperands* t, int prec, int scheme, int d, const int64_t
   if (S->tp) {
     for (int c = 0; c < 2 && d == 3; ++c)
       if ((e = alloc((void**)&S->mid[c], (size_t)kPieces * 2 * S->N)) != cudaSuccess) return e;
-    const size_t words = 4 * (2 + (size_t)tp_dep_words_max(S));
-    if ((e = alloc((void**)&S->tpctl, words)) != cudaSuccess) return e;
-    if ((e = cudaMemsetAsync(S->tpctl, 0, words, s)) != cudaSuccess) return e;
+    S->tpset = 2 + 2 * tp_slabs(S) * (int)((n[0] + 31) / 32 + 8);  // at the narrowest tiles
+    if ((e = alloc((void**)&S->tpctl, 8 * (size_t)S->tpset)) != cudaSuccess) return e;
+    if ((e = cudaMemsetAsync(S->tpctl, 0, 8 * (size_t)S->tpset, s)) != cudaSuccess) return e;
   }
   if (S->fused12 && !S->tp) {
     for (int c = 0; c < 2; ++c) {
@@ -3884,7 +3887,8 @@ cudaError_t tc_bind(TcOperands* t, adr_plan_s* P, void* u, void* v) {
   if (S->tp) {
     S->h_op.resize(np);
     for (int p = 0; p < np && e == cudaSuccess; ++p)
-      e = make_tp(S, P, S->passes[p], (float*)u, (float*)v, 1.0, S->tpctl + 2, &S->h_op[p]);
+      e = make_tp(S, P, S->passes[p], (float*)u, (float*)v, 1.0,
+                  S->tpctl + (size_t)tp_set(S, p) * S->tpset + 2, &S->h_op[p]);
     if (e != cudaSuccess) return e;
   } else {
     S->h_desc.resize(np);
@@ -3921,7 +3925,8 @@ struct GroupStep {
   const TpOp* dop;          // [np][nsolves]
   const int* tpus;          // [np][2][nsolves + 1]
   int tpnu[16][2], tpbn[16], tpchunks[16], tpnctl[16];
-  uint32_t* tpctl;
+  uint32_t* tpctl;          // two sets of tpset words
+  int tpset;
   int tpclear;              // no pointwise kernel between the operator launches
   int ring, nseg;           // 3D stencil on whole rows, 64-point segments of the widest
   PwLaunch rhs, flat;       // stencil blocks; flat pointwise blocks
@@ -3931,16 +3936,18 @@ struct GroupStep {
   double pw_n;                  // total points (pointwise statistics)
 };
 
-static cudaError_t group_step(adr_plan_s* ctl, const GroupStep& G) {
+static cudaError_t group_ops(adr_plan_s* ctl, const GroupStep& G) {
   const double N = G.pw_n;
   cudaStream_t st = ctl->stream;
-  // a pointwise kernel that writes an operator's input clears the claims of
-  // the two-pass launch that follows it
+  // The two-pass launches of a step (an even number) take the control sets in
+  // turn.  A pointwise kernel that writes an operator's input clears the set
+  // that the launch after it does not use (pw_open).
+  int set = 0;
   auto opens = [&](const PwLaunch& L) {
     PwLaunch R = L;
     R.err = G.err;
     if (G.tp) {
-      R.ctl = G.tpctl;
+      R.ctl = G.tpctl + (size_t)(set ^ 1) * G.tpset;
       for (int p = 0; p < G.np; ++p) R.nctl = std::max(R.nctl, G.tpnctl[p]);
     }
     return R;
@@ -3960,8 +3967,9 @@ static cudaError_t group_step(adr_plan_s* ctl, const GroupStep& G) {
       }
       L.nsolves = G.nsolves;
       tp_sequence(L, G.fused[p] ? 2 : 1, G.tpnu[p], G.tpchunks[p]);
-      L.ctl = G.tpctl;
+      L.ctl = G.tpctl + (size_t)set * G.tpset;
       L.nctl = G.tpnctl[p];
+      if (G.fused[p]) set ^= 1;
       L.clear = G.tpclear;
       L.err = G.err;
       e = timed_kernel(ctl, KC_MODE_TC, G.flops[p], G.bytes[p],
@@ -4053,6 +4061,13 @@ static cudaError_t group_step(adr_plan_s* ctl, const GroupStep& G) {
   return cudaSuccess;
 }
 
+static cudaError_t group_step(adr_plan_s* ctl, const GroupStep& G) {
+  const cudaError_t e = group_ops(ctl, G);
+  // a step cut short leaves a control set used and not cleared
+  if (e != cudaSuccess && G.tp) cudaMemsetAsync(G.tpctl, 0, 8 * (size_t)G.tpset, ctl->stream);
+  return e;
+}
+
 static void pass_work(const TcState* S, const TcPass& ps, double& flops, double& bytes) {
   const double N = (double)S->N, nmu = (double)S->n[ps.mu];
   const double pb = S->fmt == kFmtTF32 ? 8.0 : 6.0;  // piece bytes per value
@@ -4085,6 +4100,7 @@ static void fill_ops(GroupStep& G, const TcState* S) {
 static void fill_tp_one(GroupStep& G, const TcState* S) {
   G.hop = S->h_op.data();
   G.tpctl = S->tpctl;
+  G.tpset = S->tpset;
   for (int p = 0; p < G.np; ++p) {
     const TcPass& ps = S->passes[p];
     for (int k = 0; k < tp_npass(ps); ++k) G.tpnu[p][k] = tp_units(S, ps, k, 1.0);
@@ -4279,9 +4295,8 @@ cudaError_t tc_time_passes(TcOperands* t, adr_plan_s* P, void* u, void* v, int r
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (e == cudaSuccess) e = cudaEventCreate(&e0);
   if (e == cudaSuccess) e = cudaEventCreate(&e1);
-  // no row kernel clears the claims before the first launch
-  if (e == cudaSuccess && S->tp)
-    e = cudaMemsetAsync(S->tpctl, 0, 4 * (2 + (size_t)tp_dep_words_max(S)), P->stream);
+  // no row kernel has cleared the set of the last launch
+  if (e == cudaSuccess && S->tp) e = cudaMemsetAsync(S->tpctl, 0, 8 * (size_t)S->tpset, P->stream);
   if (e == cudaSuccess) e = cudaGraphLaunch(ge, P->stream);
   if (e == cudaSuccess) e = cudaEventRecord(e0, P->stream);
   if (e == cudaSuccess) e = cudaGraphLaunch(ge, P->stream);
@@ -4383,7 +4398,8 @@ struct adr_batch_s {
   // two-pass launches
   TpOp* d_op;           // [np][nsolves]
   int* d_tpus;          // [np][2][nsolves + 1]
-  uint32_t* d_tpctl;
+  uint32_t* d_tpctl;    // two control sets of tpset words
+  int tpset;
   std::vector<std::vector<int>> dep_at;   // [np][nsolves]: offset of a solve's counters
   int tpnu[8][2], tpbn[8], tpnctl[8];
   int ring, nseg;       // 3D stencil: whole rows if every solve's fit, segments of the widest
@@ -4630,7 +4646,7 @@ static cudaError_t batch_create_tp(adr_batch B, cudaStream_t stream, Alloc& allo
         if (k < tp_npass(ps)) acc[k] += tp_units(S, ps, k, share);
       }
       B->tpbn[p] = std::max(i ? B->tpbn[p] : 0, tp_max_bn(S, ps, share));
-      B->dep_at[p][i] = 2 + dep;
+      B->dep_at[p][i] = 2 + dep;  // within the pass's control set
       dep += tp_dep_words(S, ps, share);
     }
     for (int k = 0; k < 2; ++k) us[((size_t)p * 2 + k) * (S_ + 1) + S_] = B->tpnu[p][k] = acc[k];
@@ -4639,9 +4655,10 @@ static cudaError_t batch_create_tp(adr_batch B, cudaStream_t stream, Alloc& allo
   }
   cudaError_t e = alloc((void**)&B->d_op, sizeof(TpOp) * B->np * S_);
   if (e == cudaSuccess) e = alloc((void**)&B->d_tpus, sizeof(int) * us.size());
-  if (e == cudaSuccess) e = alloc((void**)&B->d_tpctl, sizeof(uint32_t) * words);
+  B->tpset = words;
+  if (e == cudaSuccess) e = alloc((void**)&B->d_tpctl, 8 * (size_t)words);
   if (e == cudaSuccess) e = g_upload_ring.upload(B->d_tpus, us.data(), sizeof(int) * us.size(), stream);
-  if (e == cudaSuccess) e = cudaMemsetAsync(B->d_tpctl, 0, sizeof(uint32_t) * words, stream);
+  if (e == cudaSuccess) e = cudaMemsetAsync(B->d_tpctl, 0, 8 * (size_t)words, stream);
   return e;
 }
 
@@ -4766,8 +4783,8 @@ static cudaError_t batch_bind(adr_batch B, void* const* u, void* const* v) {
       const double share = (double)S->N / B->pw_n;
       cudaError_t r = cudaSuccess;
       for (int p = 0; p < B->np && r == cudaSuccess; ++p)
-        r = make_tp(S, P, S->passes[p], (float*)u[i], (float*)v[i], share, B->d_tpctl + B->dep_at[p][i],
-                    &hop[(size_t)p * S_ + i]);
+        r = make_tp(S, P, S->passes[p], (float*)u[i], (float*)v[i], share,
+                    B->d_tpctl + (size_t)tp_set(S, p) * B->tpset + B->dep_at[p][i], &hop[(size_t)p * S_ + i]);
       if (r != cudaSuccess) return r;
     }
     cudaError_t e = make_pw(S, P, (float*)u[i], (float*)v[i], &hp[i], B->ring != 0, (double)S->N / B->pw_n);
@@ -4823,6 +4840,7 @@ static cudaError_t batch_step_direct(adr_batch B, int64_t nsteps) {
   G.dop = B->d_op;
   G.tpus = B->d_tpus;
   G.tpctl = B->d_tpctl;
+  G.tpset = B->tpset;
   G.ring = B->ring;
   G.nseg = B->nseg;
   memset(&G.rhs, 0, sizeof(G.rhs));

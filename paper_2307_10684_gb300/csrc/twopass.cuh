@@ -88,8 +88,8 @@ struct TpLaunch {
   uint32_t* ctl;             // two-pass launches: ticket, CTAs done, then the dep counters
   int nctl;                  // words to clear at the end
   int ahead;                 // units a CTA may hold claimed beyond the one it loads
-  int clear;                 // 1: no row kernel precedes: claim only after the previous kernel
-                             // has completed, and clear ctl at the end
+  int clear;                 // 1: no row kernels between the launches: claim only after the
+                             // previous kernel has completed, and clear ctl at the end
   int* err;
 };
 
@@ -210,9 +210,10 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 // which a unit reads only what earlier units write: whatever subset of the
 // grid is resident, the lowest incomplete unit is always running and never
 // waits, so the waits end without any assumption on co-residency (two plans
-// may step on two streams).  The row kernel that writes an operator's input
-// clears the counters before it lets this kernel in; a launch that follows
-// another of its kind directly (L.clear) has its last CTA do it.
+// may step on two streams).  A step's two operators have a set of counters
+// each (L.ctl); the row kernel that writes one's input clears the other's, a
+// whole kernel before that is claimed from (pw_open); a launch that follows
+// another of its kind directly (L.clear) has its last CTA clear its own.
 //
 // EPI: 0 = plain update or pieces, 1 = compensated state, 2 = the step's
 // indicators too (separate instantiations: the extra live state would cost
@@ -283,9 +284,10 @@ __global__ void __launch_bounds__(EPI == 0 ? 1024 : kTpThreads, 1) tp_kernel(con
   };
 
   if (warp == 3 && lane == 0) {
-    // ---------------- units.  The counters are cleared before this kernel
-    // is let in and only this launch adds to them, so neither the claims nor
-    // the waits for x1 tiles wait for the previous kernel
+    // ---------------- units.  The counters were cleared by a kernel that was
+    // complete before the previous one let this one in, and only this launch
+    // adds to them, so neither the claims nor the waits for x1 tiles wait for
+    // the previous kernel
     if (dynamic && L.clear) pdl_wait();
     const uint32_t* seen = nullptr;
     uint32_t t = blockIdx.x;
