@@ -3200,8 +3200,8 @@ struct PwGeom {
   int nx, ny, nz, xsegs, ytiles, zlen, zsegs;
   int64_t sy, sz;
 };
-// The 3D stencil on whole rows (rhs3_row_kernel; in a batch, if every solve's
-// rows are short enough).  us a launch, rhs3_ring_kernel / this one: 160^3
+// The 3D stencil on whole rows (rhs3_row_kernel; in a batch the solves of each
+// stencil form a part, because the two round differently).  us a launch, rhs3_ring_kernel / this one: 160^3
 // accurate mode 132 / 94, plain 45 / 40; 256^3 plain 99 / 101.
 static bool row_ring(const TcState* S) { return S->d == 3 && S->fmt == kFmtBF16 && S->n[0] <= 192; }
 static PwGeom pw_geom(const TcState* S, int num_sms, double share, bool ring) {
@@ -4402,7 +4402,7 @@ struct adr_batch_s {
   int tpset;
   std::vector<std::vector<int>> dep_at;   // [np][nsolves]: offset of a solve's counters
   int tpnu[8][2], tpbn[8], tpnctl[8];
-  int ring, nseg;       // 3D stencil: whole rows if every solve's fit, segments of the widest
+  int nseg;             // 3D stencil on whole rows: 64-point segments of the widest
   std::vector<void*> bound_u, bound_v;
   int ind_pass[8];      // per pass: some solve of the binding has indicators on
   // CUDA graph of kBatchChunk steps
@@ -4550,6 +4550,7 @@ static bool same_sequence(const adr_plan_s* a, const adr_plan_s* b) {
   if (a->prec != b->prec || (a->prec != ADR_BF16X3 && a->prec != ADR_TF32X3) || !A || !S)
     return false;
   if (S->d != A->d || S->variant != A->variant || S->fmt != A->fmt || S->scheme != A->scheme ||
+      row_ring(S) != row_ring(A) ||
       (S->comp == 2) != (A->comp == 2) ||
       S->passes.size() != A->passes.size() || S->ops.size() != A->ops.size())
     return false;
@@ -4718,19 +4719,18 @@ static adr_status batch_create_one(const adr_plan* plans, int count, void* strea
       B->units[p] = acc;
     }
     int ra = 0, rd = 0;
-    B->ring = 1;
+    const bool ring = row_ring(S0);
     B->nseg = 1;
     for (int i = 0; i < S_; ++i) {
       const TcState* S = (const TcState*)plans[i]->tc.work[0];
       B->pw_n += (double)S->N;
-      B->ring = B->ring && row_ring(S);
       B->nseg = std::max(B->nseg, (int)((S->n[0] + 63) / 64));
     }
     for (int i = 0; i < S_; ++i) {
       const TcState* S = (const TcState*)plans[i]->tc.work[0];
       bs[i] = ra;
       bs[(S_ + 1) + i] = rd;
-      ra += rhs_blocks_of(S, B->ring != 0, (double)S->N / B->pw_n);
+      ra += rhs_blocks_of(S, ring, (double)S->N / B->pw_n);
       rd += rdiff_blocks_of(S);
     }
     bs[S_] = ra;
@@ -4787,7 +4787,7 @@ static cudaError_t batch_bind(adr_batch B, void* const* u, void* const* v) {
                     B->d_tpctl + (size_t)tp_set(S, p) * B->tpset + B->dep_at[p][i], &hop[(size_t)p * S_ + i]);
       if (r != cudaSuccess) return r;
     }
-    cudaError_t e = make_pw(S, P, (float*)u[i], (float*)v[i], &hp[i], B->ring != 0, (double)S->N / B->pw_n);
+    cudaError_t e = make_pw(S, P, (float*)u[i], (float*)v[i], &hp[i], row_ring(S), (double)S->N / B->pw_n);
     if (e != cudaSuccess) return e;
   }
   for (int p = 0; p < B->np; ++p) {
@@ -4841,7 +4841,6 @@ static cudaError_t batch_step_direct(adr_batch B, int64_t nsteps) {
   G.tpus = B->d_tpus;
   G.tpctl = B->d_tpctl;
   G.tpset = B->tpset;
-  G.ring = B->ring;
   G.nseg = B->nseg;
   memset(&G.rhs, 0, sizeof(G.rhs));
   G.rhs.desc = B->d_pw;

@@ -51,6 +51,7 @@ MIXES = {
     "short_then_long": [(384, 192), (1024, 1024)],
     "long_then_short": [(1024, 1024), (384, 192)],
     "cubes": [(96, 24, 40), (160, 160, 64), (24, 96, 40), (160, 160, 64)],
+    "rows": [(64, 64, 64), (264, 40, 24), (192, 24, 40), (200, 64, 16)],  # both 3D stencils
     "slabs": [(64, 64, 96), (192, 136, 40), (64, 64, 96), (40, 200, 24)],
 }
 
