@@ -15,11 +15,14 @@
 namespace adr {
 
 // Programmatic dependent launch: a kernel of a step waits for its predecessors
-// before it touches memory, and lets the next one be scheduled when its own
-// work is nearly done.  Not at its start: the next kernel's blocks would then
-// be placed while this one's hold most SMs, several to each that is free
-// (FP64 64^2, 128 blocks a launch: 28.5 us a step so, 19.5 with the late
-// trigger, 30 without programmatic launches; 128^2 54.8 / 49.7 / 60.3).
+// before it touches memory, and lets the next one be scheduled when only its
+// own last stores are left.  Not before: the next kernel's blocks would then be
+// placed while this one's hold most SMs, several to each that is free (FP64
+// 64^2, 128 blocks a launch, us a step: trigger at the start 28.5, before the
+// epilogue 17.4, before the last stores 15.3, after them 15.8; no programmatic
+// launches 30).  Shared memory padded so that a block has its SM to itself does
+// it too (16.3), but keeps the launches of other streams off the SMs (eight
+// 64^2 solves on eight streams 64.7; 37.7 without the padding).
 __device__ __forceinline__ void simt_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void simt_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
@@ -288,7 +291,6 @@ __global__ void __launch_bounds__(C::THREADS) gemm_kernel(const __grid_constant_
           for (int j = 0; j < TN; ++j) acc[i][j] = fma(a[i][q], b[q][j], acc[i][j]);
     }
   }
-  simt_trigger();
   if constexpr (C::KS > 1) {
     static_assert(TM == 1 && TN == 1, "split contractions: one output a thread");
     __syncthreads();
@@ -319,6 +321,7 @@ __global__ void __launch_bounds__(C::THREADS) gemm_kernel(const __grid_constant_
       }
       extra[j] = x;
     }
+    if (i == TM - 1) simt_trigger();
 #pragma unroll
     for (int j = 0; j < TN; ++j) {
       const int c = n0 + col(j);
@@ -331,16 +334,12 @@ template <typename T, typename C>
 static cudaError_t run_gemm(const GemmArgs& g, cudaStream_t s) {
   const dim3 grid((g.N + C::BN - 1) / C::BN, (g.M + C::BM - 1) / C::BM, g.batch * g.ncomp);
   if (grid.y > 65535 || grid.z > 65535) return cudaErrorInvalidConfiguration;
-  // no more tiles than SMs: over half an SM's shared memory, so that no two
-  // blocks share an SM (FP64 64^2 18.0 us a step, 19.5 without)
-  constexpr int kAlone = C::SMEM > 115 * 1024 ? C::SMEM : 115 * 1024;
-  const int smem = (int64_t)grid.x * grid.y * grid.z <= 152 ? kAlone : C::SMEM;
-  if (smem > 48 * 1024) {  // an attribute of the current device's kernel, the same from every thread
+  if constexpr (C::SMEM > 48 * 1024) {  // an attribute of the kernel on the current device
     const cudaError_t e =
-        cudaFuncSetAttribute(gemm_kernel<T, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, kAlone);
+        cudaFuncSetAttribute(gemm_kernel<T, C>, cudaFuncAttributeMaxDynamicSharedMemorySize, C::SMEM);
     if (e != cudaSuccess) return e;
   }
-  return simt_launch(gemm_kernel<T, C>, grid, dim3(C::THREADS), smem, s, g);
+  return simt_launch(gemm_kernel<T, C>, grid, dim3(C::THREADS), C::SMEM, s, g);
 }
 
 // FP64: an SM retires two FMAs a clock (a warp's takes one of its four units
