@@ -380,13 +380,21 @@ static double gemm_clocks(const GemmArgs& g, double rate, double h) {
 //   512^2 361 / 131 / 109 / 97.2 / 275        1024^2 716 / 814 / 569 / 551 / 527
 //   1500^2 2203 / 2527 / 1542 / 1571 / 1365   64^3 107 / 54.4 / 47.1 / 42.9 / 79.6
 //   96^3 191 / 159 / 128 / 134 / 139          160^3 1271 / 916 / 664 / 685 / 916
+// Where an SM has one 8 x 8 tile at most, those, K split four ways as in FP64:
+// such launches are one chain of latencies.  us a step, first kernel of this
+// path / the rule above / 8 x 8:
+//   3^3 12.0 / 14.7 / 12.1    9^3 16.0 / 17.8 / 14.6    3^2 10.2 / 11.4 / 10.1
+//   32^2 13.1 / 12.0 / 10.2   64^2 17.9 / 14.2 / 10.8   300 x 8 38.0 / 21.3 / 13.7
+//   16^3 21.3 / 15.7 / 14.4
 template <>
 cudaError_t launch_gemm_simt<float>(const GemmArgs& g, cudaStream_t s) {
   if (g.M <= 0 || g.N <= 0) return cudaSuccess;
+  using S8x4 = GemmCfg<float, 8, 8, 1, 1, 64, 3, 4>;
   using S32 = GemmCfg<float, 32, 32, 2, 2, 64, 3>;
   using S64n = GemmCfg<float, 64, 32, 4, 4, 32, 3>;
   using S64 = GemmCfg<float, 64, 64, 4, 4, 32, 3>;
   using S128 = GemmCfg<float, 128, 128, 8, 8, 16, 3>;
+  if ((int64_t)((g.M + 7) / 8) * ((g.N + 7) / 8) * g.batch * g.ncomp <= 152) return run_gemm<float, S8x4>(g, s);
   const double c[4] = {gemm_clocks<S32>(g, 40.0, 0.5), gemm_clocks<S64n>(g, 62.0, 0.65),
                        gemm_clocks<S64>(g, 72.0, 0.4), gemm_clocks<S128>(g, 82.0, 0.1)};
   int best = 3;
