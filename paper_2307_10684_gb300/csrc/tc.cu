@@ -3515,35 +3515,55 @@ void tc_free(TcOperands* t) {
 
 // Whether the first two directions run as the two-pass launch (tp_kernel)
 // rather than with the intermediate in TMEM (tc_fused_kernel).  us a step,
-// tc_fused_kernel / tp_kernel, plain ETD2RKds:
+// tc_fused_kernel / tp_kernel, ETD2RKds with a plain state unless noted;
+// narrow: FHN on [0, 100]^d, wide: Brusselator on [0, 1]^d.
 //   2D  n2 <= 128, up to 32768 points (64^2 19.2 / 23.6, 128^2 25.8 / 30.4,
 //       160 x 128 27.5 / 31.2, 256 x 128 31.2 / 34.3): TMEM, one tile of x2;
-//   2D  n2 <= 256 beyond that and, with two tiles of x2, from 18000 points
-//       (Brusselator 136^2 43.3 / 34.3, 160^2 38.7 / 32.6, 200^2 49.5 / 40.6,
-//       256^2 52.5 / 39.2): two passes: a unit of tc_fused_kernel holds all of
-//       x2, and a row of tiles is one SM's work (smaller grids stay in TMEM
-//       also with two tiles, so that mixed batches of them are one launch);
+//   2D  n2 <= 128 beyond that: a unit of tc_fused_kernel is 128 rows of x1 over
+//       all of x2, so a long narrow grid still fills few SMs, but the launch
+//       is one pass.  Two passes for a compensated state (1024 x 64 52.6 / 43.9
+//       narrow, 62.7 / 51.7 wide), for rows that are no multiple of 16 (their
+//       TMA rows start off 32 bytes; 264 x 128 36.5 / 33.0 narrow, 1000 x 64
+//       33.4 / 31.9 narrow, 44.8 / 37.6 wide) unless long with narrow supports
+//       (2056 x 64 33.8 / 34.0, Lawson2b 32.3 / 34.7; wide 64.7 / 48.8), and
+//       for supports of x1 beyond 512 (2048 x 128 wide 53.0 / 50.6; Lawson2b
+//       48.6 / 50.9: not there); else TMEM (1024 x 64 27.7 / 30.8 narrow,
+//       37.4 / 38.3 wide; 2048 x 128 33.1 / 36.9 narrow);
+//   2D  n2 <= 256 and, with two tiles of x2, from 18000 points, whatever the
+//       supports (Brusselator 136^2 43.3 / 34.3, 160^2 38.7 / 32.6, 200^2
+//       49.5 / 40.6, 256^2 52.5 / 39.2; FHN narrow 136^2 42.7 / 33.2, 1024 x 136
+//       42.8 / 37.8, 2048 x 256 52.5 / 45.3): two passes (smaller grids stay in
+//       TMEM also with two tiles, so that mixed batches of them are one launch);
 //   2D  n2 > 256 and some x2 tile's support wider than the 256 intermediate
 //       columns (384^2 65.7 / 47.1, 512^2 77.0 / 53.1, 1024^2 168 / 83,
 //       FHN 2048 x 1536 160 / 132): the intermediate is computed again for
 //       every tile it reaches;
 //       narrower supports (FHN 384^2 40.0 / 40.5, 1024^2 46.0 / 54.0): TMEM;
-//   3D  up to 10^7 points (128^3 104 / 98, 160^3 281 / 188, 192^3 382 / 295),
-//       and above where 128-row tiles pad the slabs by over 10%: two passes;
+//   3D  up to 10^7 points (128^3 104 / 98, 160^3 281 / 188, 192^3 382 / 295;
+//       FHN narrow 176^3 328 / 249, 200 x 200 x 40 158 / 115, 208^3 454 / 399),
+//       and above where 128-row tiles pad the slabs by over 10% (216^3 517 / 512,
+//       264 x 200 x 264 775 / 779): two passes;
 //       256^3 (691 / 720): TMEM, whose intermediate saves HBM traffic.
-static bool tp_better(const TcState* S) {
+static bool tp_better(const TcState* S, int scheme) {
   const int64_t n1 = S->n[0], n2 = S->n[1];
+  auto widest = [&](int mu) {  // column support of a row group
+    int w = S->ksupport ? 0 : (int)S->n[mu];
+    for (int c = 0; c < 2; ++c)
+      for (int l = 0; l < 3; ++l)
+        for (const int2& r : S->hband[c][mu][l]) w = std::max(w, r.y - r.x);
+    return w;
+  };
   if (S->d == 3) {
     auto up = [](int64_t n) { return (double)((n + kBM - 1) / kBM * kBM); };
     return S->N <= 10000000 || up(n1) * up(n2) > 1.1 * (double)(n1 * n2);
   }
-  if (n2 <= kFRowsW) return n1 * n2 > (n2 > kBM ? 18000 : 32768);
-  if (!S->ksupport) return true;
-  for (int c = 0; c < 2; ++c)
-    for (int l = 0; l < 3; ++l)
-      for (const int2& r : S->hband[c][1][l])
-        if (r.y - r.x > kFRowsW) return true;
-  return false;
+  if (n2 > kFRowsW) return widest(1) > kFRowsW;
+  if (n2 > kBM) return n1 * n2 > 18000;
+  if (n1 * n2 <= 32768) return false;
+  if (S->comp) return true;
+  const int w1 = widest(0);
+  if (n1 % 16 != 0) return n1 < 2000 || w1 > kFRowsW;
+  return scheme == ADR_ETD2RKDS && w1 > 512;
 }
 
 cudaError_t tc_prepare(TcOperands* t, int prec, int scheme, int d, const int64_t n[3],
@@ -3733,7 +3753,7 @@ cudaError_t tc_prepare(TcOperands* t, int prec, int scheme, int d, const int64_t
   e = cudaStreamSynchronize(s);  // the split matrices and the supports' copies are complete
   if (e != cudaSuccess) return e;
   // no kernel requested: the library's own choice
-  S->tp = S->fused12 && variant_req < 0 && getenv("ADR_TC_VARIANT") == nullptr && tp_better(S);
+  S->tp = S->fused12 && variant_req < 0 && getenv("ADR_TC_VARIANT") == nullptr && tp_better(S, scheme);
   if (S->tp) S->variant = 0;  // one step sequence for every grid: all group in a batch
   if (S->tp) {
     for (int c = 0; c < 2 && d == 3; ++c)
