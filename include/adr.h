@@ -205,6 +205,10 @@ adr_status adr_plan_create_tuned(const adr_problem* problem, const adr_tuning* t
  * On failure the plan cannot step until a later call succeeds. */
 adr_status adr_plan_set_kernel(adr_plan plan, int32_t kernel);
 
+/* *on = 1 when the plan runs the launch of two dependent passes that only
+ * kernel -1 takes, else 0.  Host only. */
+adr_status adr_plan_two_pass(adr_plan plan, int32_t* on);
+
 /* Self-test of the bounded waits that every tensor-core and staging kernel
  * uses (no counterpart in the paper: it checks this library's failure
  * detection).  One kernel on `stream` waits on a shared-memory mbarrier
@@ -220,9 +224,11 @@ adr_status adr_selftest_bounded_wait(void* stream, int32_t arrive, int64_t limit
 
 /* Autotuner: for a tensor-core problem, builds a plan with each candidate
  * kernel, advances scratch state (allocated here, zero-filled) by 2 + nsteps
- * steps on `stream` and times the last nsteps with CUDA events.  best
- * receives the fastest of the kernels 0 to 4; ms_per_step[k] the time per step of kernel k
- * (-1 when k is not a candidate or failed).  For FP32 / FP64 problems there
+ * steps on `stream` and times the last nsteps with CUDA events.  The
+ * candidates are the kernels 0 to 4 and, on problems for which it is the
+ * launch of two dependent passes, the library's choice (-1).  best receives
+ * the fastest; ms_per_step[k] the time per step of kernel k, ms_per_step[5]
+ * that of -1 (-1 when not a candidate or failed).  For FP32 / FP64 problems there
  * is nothing to tune: best->kernel = -1 and every entry is -1.  Synchronous;
  * allocates and frees device memory.  nsteps in [1, 1024]. */
 adr_status adr_autotune(const adr_problem* problem, void* stream, int32_t nsteps,

@@ -90,6 +90,14 @@ class Plan:
         keeping the plan's matrix functions."""
         _abi.check(lib().adr_plan_set_kernel(self._p, int(kernel)))
 
+    @property
+    def two_pass(self) -> bool:
+        """adr_plan_two_pass: the plan runs the two-pass launch (kernel -1 on
+        some problems)."""
+        on = ctypes.c_int32()
+        _abi.check(lib().adr_plan_two_pass(self._p, ctypes.byref(on)))
+        return bool(on.value)
+
     def set_stream(self, stream=None):
         """adr_plan_set_stream: later calls enqueue on `stream` (default: current)."""
         self._stream = stream
@@ -316,18 +324,20 @@ _tuned = {}
 def autotune(problem, nsteps: int = 32, stream=None, cache: bool = True):
     """adr_autotune: time every tensor-core kernel variant on this problem's
     grid (scratch state, nsteps steps each) and return (best kernel, {kernel:
-    ms per step}).  Results are cached per (d, grid, precision, scheme) in
-    this process.  FP32 / FP64 problems return (-1, {})."""
-    key = (int(problem.d), tuple(int(x) for x in problem.n[: problem.d]),
-           int(problem.precision), int(getattr(problem, "scheme", 0)))
+    ms per step}); -1 is the library's choice, a candidate where that is the
+    two-pass launch.  Results are cached in this process per grid, domain,
+    diffusion, advection, step, precision, scheme and state (which decide the
+    matrices' supports, and with them the times and the library's choice).  FP32 / FP64 problems return (-1, {})."""
+    cp = make_problem(problem)
+    key = (cp.d, *cp.n, *cp.lo, *cp.hi, *cp.diff, *cp.adv[0], *cp.adv[1], cp.tau, cp.precision,
+           cp.scheme, cp.state)
     if cache and key in _tuned:
         return _tuned[key]
-    cp = make_problem(problem)
     best = _abi.AdrTuning()
     ms = (ctypes.c_float * 8)()
     _abi.check(lib().adr_autotune(ctypes.byref(cp), ctypes.c_void_p(_stream_handle(stream)),
                                   int(nsteps), ctypes.byref(best), ms))
-    out = (int(best.kernel), {k: float(ms[k]) for k in range(8) if ms[k] >= 0})
+    out = (int(best.kernel), {-1 if k == 5 else k: float(ms[k]) for k in range(6) if ms[k] >= 0})
     if cache:
         _tuned[key] = out
     return out
@@ -348,8 +358,9 @@ def autotune_batch(plans, nsteps: int = 8, stream=None):
     """Kernel choice for a batch: every tensor-core kernel is timed on the
     grouped launches of the whole batch (its plans switched with
     adr_plan_set_kernel, zero-filled scratch states, two warm-up steps, then
-    nsteps timed with CUDA events); the plans are left on the fastest kernel,
-    which is returned with {kernel: ms per step}."""
+    nsteps timed with CUDA events), and the library's own choice for each plan
+    (-1) where that is the two-pass launch for any; the plans are left on the
+    fastest kernel, which is returned with {kernel: ms per step}."""
     import torch
     plans = list(plans)
     if not plans or plans[0].precision not in (BF16X3, TF32X3):
@@ -359,9 +370,11 @@ def autotune_batch(plans, nsteps: int = 8, stream=None):
     us = [torch.zeros(pl.shape, dtype=torch.float32, device="cuda") for pl in plans]
     vs = [torch.zeros(pl.shape, dtype=torch.float32, device="cuda") for pl in plans]
     times = {}
-    for k in cands:
+    for k in cands + [-1] * (len(cands) > 1):
         for pl in plans:
             pl.set_kernel(k)
+        if k < 0 and not any(pl.two_pass for pl in plans):
+            continue  # one of the others for every plan
         b = Batch(plans, stream=st)
         b.step(us, vs, 2)
         e0 = torch.cuda.Event(enable_timing=True)

@@ -260,6 +260,8 @@ cudaError_t tc_begin_call(TcOperands* t, void* u, void* v, cudaStream_t s);
 cudaError_t tc_bind(TcOperands* t, adr_plan_s* P, void* u, void* v);
 cudaError_t tc_step(TcOperands* t, adr_plan_s* P, void* u, void* v);
 int* tc_error_word(TcOperands* t);
+// 1: the plan runs the two-pass launch.
+int tc_two_pass(const TcOperands* t);
 // Indicators of Sec. 4 accumulated by the last product of every step.
 cudaError_t tc_set_indicators(TcOperands* t, int enable, cudaStream_t s);
 cudaError_t tc_indicator_log(TcOperands* t, cudaStream_t s, double* out, int64_t max_steps,

@@ -894,15 +894,20 @@ extern "C" adr_status adr_autotune(const adr_problem* problem, void* stream, int
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   float best_ms = -1.f;
-  const int candidates[5] = {0, 1, 2, 3, 4};
-  const int ncand = prec == ADR_TF32X3 ? 1 : 5;
+  const int candidates[6] = {0, 1, 2, 3, 4, -1};
+  const int ncand = prec == ADR_TF32X3 ? 1 : 6;
   for (int c = 0; c < ncand; ++c) {
     const int k = prec == ADR_TF32X3 ? 1 : candidates[c];
+    const int slot = k < 0 ? 5 : k;
     adr_tuning t;
     memset(&t, 0, sizeof(t));
     t.kernel = k;
     adr_plan P = nullptr;
     if (adr_plan_create_tuned(problem, &t, stream, &P) != ADR_OK) continue;
+    if (k < 0 && !tc_two_pass(&P->tc)) {  // the library's choice is one of the others
+      adr_plan_destroy(P);
+      continue;
+    }
     bool ok = cudaMemsetAsync(u, 0, N * sizeof(float), s) == cudaSuccess &&
               cudaMemsetAsync(v, 0, N * sizeof(float), s) == cudaSuccess &&
               adr_step(P, u, v, 2) == ADR_OK && cudaEventRecord(e0, s) == cudaSuccess &&
@@ -920,9 +925,9 @@ extern "C" adr_status adr_autotune(const adr_problem* problem, void* stream, int
       cudaGetLastError();
       continue;
     }
-    ms_per_step[k] = ms / (float)nsteps;
-    if (best_ms < 0.f || ms_per_step[k] < best_ms) {
-      best_ms = ms_per_step[k];
+    ms_per_step[slot] = ms / (float)nsteps;
+    if (best_ms < 0.f || ms_per_step[slot] < best_ms) {
+      best_ms = ms_per_step[slot];
       best->kernel = k;
     }
   }
@@ -930,6 +935,12 @@ extern "C" adr_status adr_autotune(const adr_problem* problem, void* stream, int
   cudaEventDestroy(e1);
   cudaFree(u);
   cudaFree(v);
-  if (best->kernel < 0) return fail(ADR_EUNSUPPORTED, "adr_autotune: no kernel ran");
+  if (best_ms < 0.f) return fail(ADR_EUNSUPPORTED, "adr_autotune: no kernel ran");
+  return ADR_OK;
+}
+
+extern "C" adr_status adr_plan_two_pass(adr_plan plan, int32_t* on) {
+  if (!plan || !on) return fail(ADR_EINVAL, "NULL argument");
+  *on = tc_two_pass(&plan->tc);
   return ADR_OK;
 }

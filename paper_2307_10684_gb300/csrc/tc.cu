@@ -4382,6 +4382,11 @@ cudaError_t tc_indicator_log(TcOperands* t, cudaStream_t s, double* out, int64_t
   return cudaSuccess;
 }
 
+int tc_two_pass(const TcOperands* t) {
+  const TcState* S = (const TcState*)t->work[0];
+  return S && t->ready && S->tp;
+}
+
 int* tc_error_word(TcOperands* t) {
   TcState* S = (TcState*)t->work[0];
   return S ? S->err : nullptr;
