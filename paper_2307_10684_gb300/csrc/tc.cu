@@ -4265,10 +4265,9 @@ void tc_mode_macs(const TcOperands* t, double* dense, double* computed) {
   }
 }
 
-cudaError_t tc_time_passes(TcOperands* t, adr_plan_s* P, void* u, void* v, int reps, float* ms,
-                           int* passes) {
+static cudaError_t time_passes_bound(TcOperands* t, adr_plan_s* P, void* u, void* v, int reps, float* ms,
+                                     int* passes) {
   TcState* S = (TcState*)t->work[0];
-  if (!S || !t->ready) return cudaErrorNotSupported;
   cudaError_t e = tc_bind(t, P, u, v);
   if (e != cudaSuccess) return e;
   GroupStep G;
@@ -4328,6 +4327,38 @@ cudaError_t tc_time_passes(TcOperands* t, adr_plan_s* P, void* u, void* v, int r
   if (e0) cudaEventDestroy(e0);
   if (e1) cudaEventDestroy(e1);
   if (ge) cudaGraphExecDestroy(ge);
+  return e;
+}
+// The timed launches run with low-order words and indicator sums of their own:
+// the plan's belong to the state that it steps (and before the first step the
+// indicator slot is -1).
+cudaError_t tc_time_passes(TcOperands* t, adr_plan_s* P, void* u, void* v, int reps, float* ms,
+                           int* passes) {
+  TcState* S = (TcState*)t->work[0];
+  if (!S || !t->ready) return cudaErrorNotSupported;
+  float* lo[2] = {S->lo[0], S->lo[1]};
+  double* ind = S->ind;
+  int64_t* ctr = S->ind_ctr;
+  const size_t slots = ind ? sizeof(double) * 4 * kIndSlots : 0;
+  const size_t words = S->comp ? sizeof(float) * S->N : 0, bytes = 2 * words + slots + sizeof(int64_t);
+  uint8_t* own = nullptr;
+  cudaError_t e = cudaMalloc((void**)&own, bytes);
+  if (e != cudaSuccess) return e;
+  e = cudaMemsetAsync(own, 0, bytes, P->stream);
+  if (ind) {
+    S->ind = (double*)(own + 2 * words);
+    S->ind_ctr = (int64_t*)(own + 2 * words + slots);
+  }
+  for (int c = 0; c < 2 && S->comp; ++c) S->lo[c] = (float*)(own + c * words);
+  S->bound_u = S->bound_v = nullptr;
+  if (e == cudaSuccess) e = time_passes_bound(t, P, u, v, reps, ms, passes);
+  S->ind = ind;
+  S->ind_ctr = ctr;
+  S->lo[0] = lo[0];
+  S->lo[1] = lo[1];
+  S->bound_u = S->bound_v = nullptr;  // descriptors are rebuilt at the next bind
+  cudaStreamSynchronize(P->stream);
+  cudaFree(own);
   return e;
 }
 
