@@ -1570,10 +1570,10 @@ __device__ __forceinline__ void split3_pair(float x0, float x1, uint32_t& w0, ui
   const float r0 = x0 - f0.x, r1 = x1 - f0.y;
   const __nv_bfloat162 h1 = __floats2bfloat162_rn(r0, r1);
   const float2 f1 = __bfloat1622float2(h1);
-  const __nv_bfloat162 tp = __floats2bfloat162_rn(r0 - f1.x, r1 - f1.y);
+  const __nv_bfloat162 h2 = __floats2bfloat162_rn(r0 - f1.x, r1 - f1.y);
   w0 = *reinterpret_cast<const uint32_t*>(&h0);
   w1 = *reinterpret_cast<const uint32_t*>(&h1);
-  w2 = *reinterpret_cast<const uint32_t*>(&tp);
+  w2 = *reinterpret_cast<const uint32_t*>(&h2);
 }
 static_assert(2 * kPieces * kFTileC <= kFStage, "an MMA2 stage fits in a ring slot");
 static_assert(kFSmem <= 227 * 1024, "shared memory per CTA");
@@ -2986,8 +2986,7 @@ cudaError_t launch_rhs3_rows(int nseg, int blocks, cudaStream_t s, const PwLaunc
   const dim3 g(blocks), b(kPwThreads);
   if (nseg == 1) return launch_k(rhs3_row_kernel<1, DF>, g, b, kRowRingSmem, s, L);
   if (nseg == 2) return launch_k(rhs3_row_kernel<2, DF>, g, b, kRowRingSmem, s, L);
-  if (nseg == 3) return launch_k(rhs3_row_kernel<3, DF>, g, b, kRowRingSmem, s, L);
-  return launch_k(rhs3_row_kernel<4, DF>, g, b, kRowRingSmem, s, L);
+  return launch_k(rhs3_row_kernel<3, DF>, g, b, kRowRingSmem, s, L);
 }
 cudaError_t set_tp_attr() {
   const auto at = cudaFuncAttributeMaxDynamicSharedMemorySize;
@@ -3010,11 +3009,9 @@ cudaError_t set_tp_attr() {
   set(rhs3_row_kernel<1, false>, kRowRingSmem);
   set(rhs3_row_kernel<2, false>, kRowRingSmem);
   set(rhs3_row_kernel<3, false>, kRowRingSmem);
-  set(rhs3_row_kernel<4, false>, kRowRingSmem);
   set(rhs3_row_kernel<1, true>, kRowRingSmem);
   set(rhs3_row_kernel<2, true>, kRowRingSmem);
   set(rhs3_row_kernel<3, true>, kRowRingSmem);
-  set(rhs3_row_kernel<4, true>, kRowRingSmem);
   return e;
 }
 
@@ -3201,9 +3198,10 @@ struct PwGeom {
   int64_t sy, sz;
 };
 // The 3D stencil on whole rows (rhs3_row_kernel; in a batch the solves of each
-// stencil form a part, because the two round differently).  us a launch, rhs3_ring_kernel / this one: 160^3
-// accurate mode 132 / 94, plain 45 / 40; 256^3 plain 99 / 101.
-static bool row_ring(const TcState* S) { return S->d == 3 && S->fmt == kFmtBF16 && S->n[0] <= 192; }
+// stencil form a part, because the two round differently).  us a launch,
+// rhs3_ring_kernel / this one: 160^3 accurate mode 132 / 94, plain 45 / 40;
+// 256^3 plain 99 / 101.
+static bool row_ring(const TcState* S) { return S->d == 3 && S->fmt == kFmtBF16 && S->n[0] <= kRowRingX; }
 static PwGeom pw_geom(const TcState* S, int num_sms, double share, bool ring) {
   PwGeom g;
   const bool d3 = S->d == 3;

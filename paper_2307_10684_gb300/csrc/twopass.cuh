@@ -633,7 +633,7 @@ __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
       : "memory");
   return ok != 0;
 }
-// 3D stencil and reaction for rows of up to 256 points.  A block owns 8 rows
+// 3D stencil and reaction for rows of up to 192 points.  A block owns 8 rows
 // (y0 .. y0 + 7), one per warp, and marches zlen planes.  Each plane of u and
 // v (its 8 rows and the two beside them) arrives by one TMA copy per field
 // into a ring of shared-memory slots; a row's own values stay in registers
@@ -644,7 +644,8 @@ __device__ __forceinline__ bool mbar_test_wait(uint64_t* bar, uint32_t parity) {
 // lanes idle than four points a lane would.
 constexpr int kRowRingY = 8;
 static_assert(kRowRingY == kPwWarps, "one row per warp");
-constexpr int kRowRingField = 256 * (kRowRingY + 2);   // floats per field and plane
+constexpr int kRowRingX = 192;
+constexpr int kRowRingField = kRowRingX * (kRowRingY + 2);   // floats per field and plane
 constexpr int kRowRingSlots = 5;
 constexpr int kRowRingSmem = kRowRingSlots * 2 * kRowRingField * 4 + 128 + 2 * kRowRingSlots * 8;
 // The x direction at point j of a pair starting at an even index, on a row of
