@@ -4092,6 +4092,7 @@ static void pass_work(const TcState* S, const TcPass& ps, double& flops, double&
   flops = 2.0 * 2.0 * nmu * N;
   if (ps.fused) flops = 2.0 * 2.0 * (double)(S->n[0] + S->n[1]) * N;  // two products
   bytes = 2.0 * (pb * N + pb * nmu * nmu);
+  if (ps.tp && ps.fused) bytes += 2.0 * 2.0 * pb * N;  // the intermediate out and in
   if (ps.mode == kPieces3) bytes += 2.0 * pb * N;
   if (ps.mode == kAxpy) bytes += 2.0 * (S->comp ? 16.0 : 8.0) * N;  // base, out (+ lo in, out)
   if (ps.mode == kStage1 || ps.mode == kStage1X) bytes += 2.0 * (8.0 + pb) * N;
