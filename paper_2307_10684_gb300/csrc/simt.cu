@@ -352,6 +352,8 @@ static cudaError_t run_gemm(const GemmArgs& g, cudaStream_t s) {
 //   32^3 60.5 / 46.0 / 51.2   64^3 415 / 403 / 414      160^3 17024 / 13469 / 13677
 // (16 x 16 tiles: 48.8, 280, 1835, 13917; 45.3, 403, 13330.)  What is left
 // above the FMA time (256^2: 232 us) is the pointwise kernels and launches.
+// (Measured with an earlier trigger; with the present one, above, 32^2 12.8,
+// 64^2 15.3, 128^2 45.3.)
 template <>
 cudaError_t launch_gemm_simt<double>(const GemmArgs& g, cudaStream_t s) {
   if (g.M <= 0 || g.N <= 0) return cudaSuccess;

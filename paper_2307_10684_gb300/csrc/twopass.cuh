@@ -23,8 +23,9 @@
 // N / 2 beyond (measured: 48 ns apart at N = 32, 80 and 128).  So of tiles that
 // contract over the same range the widest is the cheapest per output: 136^3
 // runs at 145 us a step with one tile of 144 columns, 163 with two of 80
-// (192^3 296 / 312; 160^3 190 / 185, whose epilogues overlap better).  Beyond
-// 256 columns 128-wide tiles with ranges of their own win, and narrower tiles
+// (192^3 296 / 312; 160^3 190 / 185, where a tile's latencies bound: the
+// tensor pipe is busy 28% of the launch, no memory above 36%).  Beyond 256
+// columns 128-wide tiles with ranges of their own win, and narrower tiles
 // serve to spread small grids over more SMs (tp_geo).
 
 constexpr int kTpBK = 32;                          // K values per stage (64-byte rows)
